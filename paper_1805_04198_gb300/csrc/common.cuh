@@ -84,17 +84,33 @@ __device__ __forceinline__ T local_solve2(T vmx, T vpx, T vmy, T vpy, T rh, uint
 }
 
 // Value-only variant used inside the sweeps (the wind is recomputed from the
-// converged state, so the sweeps need only the value).
+// converged state, so the sweeps need only the value), from the axis minima.
+// The two-term branch needs no clamp of the discriminant: where it is taken,
+// |a - b| < r h, the discriminant is at least (r h)^2; where it is negative or
+// NaN its root is not selected.  In FP64 the root of an unselected
+// discriminant is kept off the square root's slow path.
+__device__ __forceinline__ float local_solve2_min(float a, float b, float rh) {
+    using N = Num<float>;
+    const float d = N::sub(a, b);
+    const float disc = N::sub(N::mul(N::mul(2.f, rh), rh), N::mul(d, d));
+    // (a + b + root) / 2 as one rounding of root / 2 + (a + b) / 2: halving is
+    // exact, so this is the same value with a shorter chain behind the root
+    const float u2 = __fmaf_rn(N::sqrt_solve(disc), 0.5f, N::mul(N::add(a, b), 0.5f));
+    const float u1 = N::add(fmin(a, b), rh);
+    return fabsf(d) < rh ? u2 : u1;
+}
+__device__ __forceinline__ double local_solve2_min(double a, double b, double rh) {
+    using N = Num<double>;
+    const double d = N::sub(a, b);
+    const bool two = fabs(d) < rh;
+    const double disc = N::sub(N::mul(N::mul(2.0, rh), rh), N::mul(d, d));
+    const double u2 = N::mul(N::add(N::add(a, b), N::sqrt_solve(two ? disc : 1.0)), 0.5);
+    const double u1 = N::add(fmin(a, b), rh);
+    return two ? u2 : u1;
+}
 template <class T>
 __device__ __forceinline__ T local_solve2_value(T vmx, T vpx, T vmy, T vpy, T rh) {
-    using N = Num<T>;
-    const T a = fmin(vmx, vpx);
-    const T b = fmin(vmy, vpy);
-    const T d = N::sub(a, b);
-    const T disc = N::sub(N::mul(N::mul(T(2), rh), rh), N::mul(d, d));
-    const T u2 = N::mul(N::add(N::add(a, b), N::sqrt_solve(fmax(disc, T(0)))), T(0.5));
-    const T u1 = N::add(fmin(a, b), rh);
-    return fabs(d) < rh ? u2 : u1;
+    return local_solve2_min(fmin(vmx, vpx), fmin(vmy, vpy), rh);
 }
 
 // 3-D Godunov local solve: axis minima sorted a_p0 <= a_p1 <= a_p2 (ties keep

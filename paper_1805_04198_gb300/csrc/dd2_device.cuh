@@ -85,34 +85,21 @@ __device__ __forceinline__ T fine_at(const T *a, long long sy, int X, int Y) {
 // Engine policies
 // --------------------------------------------------------------------------
 
-// FSM update u = min(u, u~) (Sec. 1.1, eq. FSMupdate).  Statics: r, stored
-// as a non-positive value at fixed nodes (Gamma).
-template <class T>
-struct FsmPolicy {
-    T h;
-    __device__ __forceinline__ T update(T self, T vmx, T vpx, T vmy, T vpy, const T *sv, uint8_t,
-                                        bool &changed) const {
-        const T r = sv[0];
-        const T ut = local_solve2_value(vmx, vpx, vmy, vpy, Num<T>::mul(r, h));
-        const bool take = (r > T(0)) && (ut < self);
-        changed = take;
-        return take ? ut : self;
-    }
-};
-
-// Alg. 5 weighted correction.  Statics: r, u^k, C_H(nbrs U^k); byte mask:
-// bit 0 Gamma, bits 1/2 "x component may be <= 0 / >= 0", bits 3/4 the same
+// Alg. 5 weighted correction.  Statics: r H, u^k, C_H(nbrs U^k); byte mask:
+// bit 0 fixed (Gamma, or outside the grid: the value is kept), bits 1/2 "x component may be <= 0 / >= 0", bits 3/4 the same
 // for y (from w^k and W^k on the axes of the node's coarse lines; both set on
 // other axes).
 template <class T>
 struct Alg5Policy {
-    T H, theta;
+    static constexpr bool SYM = false;
+    static __device__ __forceinline__ T pad() { return Num<T>::inf(); }
+    T theta;
     bool per_node;  // weight from the fourth static instead of `theta`
     __device__ __forceinline__ T update(T self, T vmx, T vpx, T vmy, T vpy, const T *sv, uint8_t mask,
                                         bool &changed) const {
         using N = Num<T>;
         uint8_t w;
-        const T Ut = local_solve2(vmx, vpx, vmy, vpy, N::mul(sv[0], H), w);
+        const T Ut = local_solve2(vmx, vpx, vmy, vpy, sv[0], w);
         const T uk = sv[1], cold = sv[2];
         const int wx = wind_comp(w, 0), wy = wind_comp(w, 1);
         bool pass = (Ut < N::inf()) && (cold < N::inf());
@@ -131,20 +118,30 @@ struct Alg5Policy {
 // --------------------------------------------------------------------------
 // Bodies take the block index and count explicitly so that the batched
 // kernels (several problems per launch) can reuse them.
+// The statics are written in storage order, 16 bytes per thread (positions
+// outside the box included, with the value that keeps them inert).
 template <class T>
 __device__ void pack_tiles_body(const DDArgs<T> &A, size_t bid, size_t nbid) {
+    constexpr int E = 16 / (int)sizeof(T);
     const DDGeom &G = A.G;
-    const size_t per_tile = (size_t)G.tnx * G.tny;
+    const size_t per_tile = G.tile_sk_elems / E;
     const size_t total = per_tile * G.tx * G.ty;
+    const T hs = T(G.h);
     for (size_t t = bid * blockDim.x + threadIdx.x; t < total; t += nbid * blockDim.x) {
-        int tile = (int)(t / per_tile);
-        int rem = (int)(t % per_tile);
-        int xl = rem % G.tnx, yl = rem / G.tnx;
-        int tx = tile % G.tx, ty = tile / G.tx;
-        int X = tx * G.sx + xl, Y = ty * G.sy + yl;
-        T v = A.gamma[(size_t)Y * A.sy + X] ? T(-1) : fine_at(A.r, A.sy, X, Y);
-        T *base = A.tile_rsk + (size_t)tile * G.tile_sk_elems;
-        for (int d = 0; d < 4; ++d) base[skew_index(d, xl, yl, G.tnb, G.tny, G.tnstepp)] = v;
+        const int tile = (int)(t / per_tile);
+        const size_t e0 = (t - tile * per_tile) * E;
+        const int tx = tile % G.tx, ty = tile / G.tx;
+        union { T v[E]; uint4 w; } o;
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            int xl, yl;
+            o.v[i] = Num<T>::inf();
+            if (skew_node<T>(e0 + i, G.tnx, G.tny, G.tnb, G.tnstepp, xl, yl)) {
+                const size_t f = (size_t)(ty * G.sy + yl) * A.sy + tx * G.sx + xl;
+                o.v[i] = FsmPolicy<T>::node(A.gamma[f] != 0, A.r[f], hs);
+            }
+        }
+        reinterpret_cast<uint4 *>(A.tile_rsk)[t] = o.w;
     }
 }
 
@@ -155,20 +152,47 @@ __global__ void k_pack_tiles(DDArgs<T> A) {
 
 template <class T>
 __device__ void pack_coarse_body(const DDArgs<T> &A, size_t bid, size_t nbid) {
+    constexpr int E = 16 / (int)sizeof(T);
     const DDGeom &G = A.G;
     for (size_t a = bid * blockDim.x + threadIdx.x; a < G.coarse_elems; a += nbid * blockDim.x) {
         int g, i, j;
-        if (!coarse_decode(G, a, g, i, j)) continue;
+        if (!coarse_decode(G, a, g, i, j)) {  // padding columns
+            A.U0[a] = Num<T>::inf();
+            continue;
+        }
         GridDesc d = grid_desc(G, g);
         int X = d.ox + G.c * i, Y = d.oy + G.c * j;
         bool gam = A.gamma[(size_t)Y * A.sy + X] != 0;
-        T rv = fine_at(A.r, A.sy, X, Y);
-        A.rc[a] = gam ? T(-1) : rv;
+        A.rc[a] = gam ? T(-1) : fine_at(A.r, A.sy, X, Y);
         A.U0[a] = gam ? fine_at(A.g, A.sy, X, Y) : Num<T>::inf();
         A.W[a] = WIND_ZERO;
-        T *sk = A.rc_sk + d.skoff;
-        for (int dd = 0; dd < 4; ++dd) sk[skew_index(dd, i, j, d.nb, d.my, d.nstepp)] = gam ? T(-1) : rv;
     }
+    const size_t nv = G.coarse_sk_elems / E;
+    const T Hs = T(G.H);
+    for (size_t t = bid * blockDim.x + threadIdx.x; t < nv; t += nbid * blockDim.x) {
+        const size_t a0 = t * E;
+        int g = 0;
+        if (a0 >= G.k0) {
+            const size_t t1 = a0 - G.k0, hk = (size_t)(G.c - 1) * G.kh;
+            g = t1 < hk ? 1 + (int)(t1 / G.kh) : G.c + (int)((t1 - hk) / G.kv);
+        }
+        const GridDesc d = grid_desc(G, g);
+        union { T v[E]; uint4 w; } o;
+#pragma unroll
+        for (int q = 0; q < E; ++q) {
+            int i, j;
+            o.v[q] = Num<T>::inf();
+            if (skew_node<T>(a0 - d.skoff + q, d.mx, d.my, d.nb, d.nstepp, i, j)) {
+                const size_t f = (size_t)(d.oy + G.c * j) * A.sy + d.ox + G.c * i;
+                o.v[q] = FsmPolicy<T>::node(A.gamma[f] != 0, A.r[f], Hs);
+            }
+        }
+        reinterpret_cast<uint4 *>(A.rc_sk)[t] = o.w;
+    }
+    // positions outside a grid are kept as they are by the Alg. 5 sweeps
+    if (!A.step4_identity)
+        for (size_t t = bid * blockDim.x + threadIdx.x; t < G.coarse_sk_elems / 16; t += nbid * blockDim.x)
+            reinterpret_cast<uint4 *>(A.mask_sk)[t] = make_uint4(0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u);
 }
 
 template <class T>
@@ -217,11 +241,10 @@ __device__ __forceinline__ void k_step1_body(const DDArgs<T> &A, char *smem, int
     bx.u = A.U + d.off;
     bx.st[0] = A.rc_sk + d.skoff;
     bx.sb = nullptr;
-    bx.nx = d.mx;
     bx.ny = d.my;
     bx.nb = d.nb;
     bx.nstepp = d.nstepp;
-    FsmPolicy<T> pol{T(G.H)};
+    FsmPolicy<T> pol;
     long long sweeps;
     bool conv;
     engine_run<T, 1, false>(bx, pol, A.max_coarse, smem, sweeps, conv, &A.st->err);
@@ -239,7 +262,6 @@ __device__ __forceinline__ void k_step4_gen(const DDArgs<T> &A, char *smem, int 
     if (*A.done || A.step4_identity) return;  // weight 0: Alg. 4 already wrote U^{k+1} = u^k
     const DDGeom &G = A.G;
     const GridDesc d = grid_desc(G, gidx);
-    const T Hs = T(G.H);
     const size_t n = (size_t)d.nb * d.my * 32;
     T *U = A.U + d.off;
     // C_H(nbrs^H(U^k)), U^k and W = w^k were prepared by Alg. 4 (alg4_body)
@@ -255,11 +277,10 @@ __device__ __forceinline__ void k_step4_gen(const DDArgs<T> &A, char *smem, int 
     bx.st[2] = A.cold_sk + d.skoff;
     if (ADAPT) bx.st[NST - 1] = A.theta_sk + d.skoff;
     bx.sb = A.mask_sk + d.skoff;
-    bx.nx = d.mx;
     bx.ny = d.my;
     bx.nb = d.nb;
     bx.nstepp = d.nstepp;
-    Alg5Policy<T> pol{Hs, A.theta, ADAPT};
+    Alg5Policy<T> pol{A.theta, ADAPT};
     long long sweeps;
     bool conv;
     engine_run<T, NST, true>(bx, pol, A.max_coarse, smem, sweeps, conv, &A.st->err);
@@ -609,7 +630,7 @@ __device__ bool tile_needs_solve(const DDArgs<T> &A, int tile) {
     return need;
 }
 
-template <class T, bool STEADY_PATH = true>
+template <class T>
 __device__ __forceinline__ void k_fine_body(const DDArgs<T> &A, char *smem, int tile, bool check = true) {
     if (*A.done) return;
     if (check && !tile_needs_solve(A, tile)) {
@@ -636,8 +657,8 @@ __device__ __forceinline__ void k_fine_body(const DDArgs<T> &A, char *smem, int 
         }
         ut[e] = v;
     }
-    // (Gamma nodes carry a non-positive slowness in the skewed statics, set
-    // once when the statics are packed)
+    // (Gamma nodes carry an infinite r h in the skewed statics, set once when
+    // the statics are packed)
     __threadfence_block();
     __syncthreads();
     // Step 3: FSM sweeps in the subdomain
@@ -645,14 +666,13 @@ __device__ __forceinline__ void k_fine_body(const DDArgs<T> &A, char *smem, int 
     bx.u = ut;
     bx.st[0] = A.tile_rsk + (size_t)tile * G.tile_sk_elems;
     bx.sb = nullptr;
-    bx.nx = NX;
     bx.ny = NY;
     bx.nb = G.tnb;
     bx.nstepp = G.tnstepp;
-    FsmPolicy<T> pol{T(G.h)};
+    FsmPolicy<T> pol;
     long long sweeps;
     bool conv;
-    engine_run<T, 1, false, false, STEADY_PATH>(bx, pol, A.max_fsm, smem, sweeps, conv, &A.st->err);
+    engine_run<T, 1, false>(bx, pol, A.max_fsm, smem, sweeps, conv, &A.st->err);
     if (threadIdx.x == 0) {
         atomicMax(&A.st->fsm_sweeps_max, (unsigned long long)sweeps);
         if (!conv) atomicAdd(&A.st->fsm_caps, 1ull);
@@ -872,9 +892,9 @@ __device__ void alg4_body(const DDArgs<T> &A, int k, size_t bid, size_t nbid) {
             th = (T)thv;
         }
         for (int dd = 0; dd < 4; ++dd) {
-            size_t si = d.skoff + skew_index(dd, i, j, d.nb, d.my, d.nstepp);
+            const size_t si = d.skoff + skew_index<T>(dd, i, j, d.nb, d.my, d.nstepp);
             A.uk_sk[si] = ukv;
-            A.mask_sk[si] = m;
+            A.mask_sk[d.skoff + skew_index<uint8_t>(dd, i, j, d.nb, d.my, d.nstepp)] = m;
             A.cold_sk[si] = cold;
             if (A.theta_sk) A.theta_sk[si] = th;  // per-node or (in a mixed batch) constant weight
         }

@@ -13,6 +13,7 @@ struct DDPlan {
     DDGeom G;
     size_t bytes;
     size_t fine_smem, step1_smem, step4_smem;
+    size_t fine_limit, step1_limit, step4_limit;  // what decides whether the size is supported
     int grid_threads;
     bool adaptive;  // per-node weight: history of C_H and a fourth Alg. 5 static
 };
@@ -140,17 +141,18 @@ inline DDPlan dd_plan(const eik_grid *grid, const eik_dd_params *p) {
                                      : dd_layout<float>(P, nullptr, nullptr, p->max_iter);
     const int gnb = ceil32(P.G.ncx + 1);
     P.grid_threads = 32 * gnb;
-    if (grid->dtype == EIK_F64) {
-        P.fine_smem = engine_smem_bytes<double, 1, false>(P.G.tnb, P.G.tny);
-        P.step1_smem = engine_smem_bytes<double, 1, false>(gnb, P.G.ncy + 1);
-        P.step4_smem = P.adaptive ? engine_smem_bytes<double, 4, true>(gnb, P.G.ncy + 1)
-                                  : engine_smem_bytes<double, 3, true>(gnb, P.G.ncy + 1);
-    } else {
-        P.fine_smem = engine_smem_bytes<float, 1, false>(P.G.tnb, P.G.tny);
-        P.step1_smem = engine_smem_bytes<float, 1, false>(gnb, P.G.ncy + 1);
-        P.step4_smem = P.adaptive ? engine_smem_bytes<float, 4, true>(gnb, P.G.ncy + 1)
-                                  : engine_smem_bytes<float, 3, true>(gnb, P.G.ncy + 1);
-    }
+    auto sizes = [&](auto zero) {
+        using T = decltype(zero);
+        const int my = P.G.ncy + 1;
+        P.fine_smem = engine_smem_bytes<T, 1, false>(P.G.tnb, P.G.tny);
+        P.step1_smem = engine_smem_bytes<T, 1, false>(gnb, my);
+        P.step4_smem = P.adaptive ? engine_smem_bytes<T, 4, true>(gnb, my) : engine_smem_bytes<T, 3, true>(gnb, my);
+        P.fine_limit = engine_limit_bytes<T, 1, false>(P.G.tnb, P.G.tny);
+        P.step1_limit = engine_limit_bytes<T, 1, false>(gnb, my);
+        P.step4_limit = P.adaptive ? engine_limit_bytes<T, 4, true>(gnb, my) : engine_limit_bytes<T, 3, true>(gnb, my);
+    };
+    if (grid->dtype == EIK_F64) sizes(0.0);
+    else sizes(0.f);
     return P;
 }
 

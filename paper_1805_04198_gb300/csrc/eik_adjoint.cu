@@ -53,6 +53,7 @@ struct AdjArgs {
     AdjDev *dev;
     long long max_sweeps;
     int launches;
+    int multi;  // multi-CTA form
 };
 
 // dF_j/du of node j towards each neighbour side and dF_j/dr_j (zero where j
@@ -127,40 +128,34 @@ __global__ void k_adj_nodes(AdjArgs<T> A) {
     adj_nodes_body(A, blockIdx.x, gridDim.x);
 }
 
-// Skewed statics in output order: thread e writes element e of every channel
-// ([dir][logical block][step][lane], the inverse of skew_index), so a warp's
-// stores are contiguous; positions outside the box get 0.
+// Skewed statics in storage order, 16 bytes of every channel per thread
+// ([dir][logical block][stream], see skew_index); positions outside the box
+// get 0, and so does the state.  For the multi-CTA form also the empty
+// hand-off columns.
 template <class T>
 __device__ void adj_pack_body(const AdjArgs<T> &A, size_t bid, size_t nbid) {
+    constexpr int E = 16 / (int)sizeof(T);
     const size_t n = (size_t)A.nx * A.ny;
     const size_t chan = (size_t)4 * A.nb * A.nstepp * 32;
-    for (size_t e = bid * blockDim.x + threadIdx.x; e < chan; e += nbid * blockDim.x) {
-        const int l = (int)(e & 31);
-        const size_t row = e >> 5;
-        const int st = (int)(row % A.nstepp);
-        const int q = (int)((row / A.nstepp) % A.nb);
-        const int d = (int)(row / ((size_t)A.nstepp * A.nb));
-        const int sx = dir_sx(d), sy = dir_sy(d);
-        const int x = 32 * (sx > 0 ? q : A.nb - 1 - q) + (sx > 0 ? l : 31 - l);
-        const int lr = st - l;
-        T v0 = T(0), v1 = T(0), v2 = T(0), v3 = T(0), v4 = T(0);
-        if (x < A.nx && lr >= 0 && lr < A.ny) {
-            const int y = sy > 0 ? lr : A.ny - 1 - lr;
-            const size_t t = (size_t)y * A.nx + x;
-            v0 = A.win[t];
-            v1 = A.win[n + t];
-            v2 = A.win[2 * n + t];
-            v3 = A.win[3 * n + t];
-            v4 = A.dJdu[(size_t)y * A.sy + x];
+    for (size_t t = bid * blockDim.x + threadIdx.x; t < chan / E; t += nbid * blockDim.x) {
+        union { T v[E]; uint4 w; } o[5];
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            int x, y;
+            const bool in = skew_node<T>(t * E + i, A.nx, A.ny, A.nb, A.nstepp, x, y);
+            const size_t j = in ? (size_t)y * A.nx + x : 0;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) o[c].v[i] = in ? A.win[c * n + j] : T(0);
+            o[4].v[i] = in ? A.dJdu[(size_t)y * A.sy + x] : T(0);
         }
-        A.sk[e] = v0;
-        A.sk[chan + e] = v1;
-        A.sk[2 * chan + e] = v2;
-        A.sk[3 * chan + e] = v3;
-        A.sk[4 * chan + e] = v4;
+#pragma unroll
+        for (int c = 0; c < 5; ++c) reinterpret_cast<uint4 *>(A.sk + c * chan)[t] = o[c].w;
     }
     const size_t box = (size_t)A.nb * A.ny * 32;
     for (size_t t = bid * blockDim.x + threadIdx.x; t < box; t += nbid * blockDim.x) A.state[t] = T(0);
+    if (A.multi)
+        for (size_t t = bid * blockDim.x + threadIdx.x; t < A.nb * hand_elems(A.ny); t += nbid * blockDim.x)
+            A.ghands[t] = Hand<T>::empty();
 }
 
 template <class T>
@@ -171,6 +166,8 @@ __global__ void k_adj_pack(AdjArgs<T> A) {
 // lambda_i = dJ/du_i + W(-x) l(-x) + W(+x) l(+x) + W(-y) l(-y) + W(+y) l(+y)
 template <class T>
 struct AdjPolicy {
+    static constexpr bool SYM = false;
+    static __device__ __forceinline__ T pad() { return T(0); }  // its weight is 0
     __device__ __forceinline__ T update(T self, T vmx, T vpx, T vmy, T vpy, const T *sv, uint8_t,
                                         bool &changed) const {
         using N = Num<T>;
@@ -191,7 +188,6 @@ __device__ __forceinline__ Box<T, 5> adj_box(const AdjArgs<T> &A) {
     bx.u = A.state;
     for (int c = 0; c < 5; ++c) bx.st[c] = A.sk + c * chan;
     bx.sb = nullptr;
-    bx.nx = A.nx;
     bx.ny = A.ny;
     bx.nb = A.nb;
     bx.nstepp = A.nstepp;
@@ -279,7 +275,7 @@ static size_t adj_layout(const AdjPlan &P, AdjArgs<T> *A, void *ws) {
     T *dudr = cv.take<T>(n);
     T *state = cv.take<T>((size_t)P.nb * P.ny * 32);
     T *sk = cv.take<T>((size_t)5 * 4 * P.nb * P.nstepp * 32);
-    T *ghands = cv.take<T>((size_t)P.nb * P.ny);
+    T *ghands = cv.take<T>(P.nb * hand_elems(P.ny));
     int *gctl = cv.take<int>(engine_global_ints(P.nb));
     AdjDev *dev = cv.take<AdjDev>(1);
     if (A) {
@@ -340,6 +336,7 @@ static int adj_run(const eik_grid *grid, const AdjPlan &P, const void *r, const 
     if ((rc = cuda_check(cudaFuncGetAttributes(&fa, k_adj_run<T>), "func attr"))) return rc;
     const bool single = (int)P.smem <= optin && P.nb <= 32 && regs_fit(fa, P.nb);
     A.launches = single ? 5 : 6;
+    A.multi = single ? 0 : 1;
     const size_t total = (size_t)P.nx * P.ny;
     const int tb = (int)std::min<size_t>((total + 255) / 256, (size_t)nsm * 16);
     EIK_LAUNCH("adj_zero", s, k_adj_zero<T><<<tb, 256, 0, s>>>(A));
@@ -551,6 +548,7 @@ static int adj_many_run(const eik_grid *grid, const AdjManyPlan &MP, int nprob, 
     const int ngroups = (nprob + group - 1) / group;
     nl += 4 + (single ? 1 : 1 + ngroups) + (grad_sum ? 1 : 0);
     A.launches = nl;
+    A.multi = single ? 0 : 1;
     const size_t total = (size_t)P.nx * P.ny;
     const dim3 eg((unsigned)std::max<size_t>(1, std::min<size_t>((total + 255) / 256, (size_t)nsm * 16 / nprob + 1)),
                   (unsigned)nprob);

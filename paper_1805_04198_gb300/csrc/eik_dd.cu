@@ -238,9 +238,9 @@ struct DDSolve {
         cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         fine_threads = 32 * G.tnb;
         fine_smem = P.fine_smem;
-        if ((int)fine_smem > smem_optin || (int)P.step1_smem > smem_optin || (int)P.step4_smem > smem_optin) {
-            set_error("shared memory need (%zu, %zu, %zu) exceeds the device limit %d", fine_smem, P.step1_smem,
-                      P.step4_smem, smem_optin);
+        if ((int)P.fine_limit > smem_optin || (int)P.step1_limit > smem_optin || (int)P.step4_limit > smem_optin) {
+            set_error("shared memory need (%zu, %zu, %zu) exceeds the device limit %d", P.fine_limit, P.step1_limit,
+                      P.step4_limit, smem_optin);
             return EIK_EUNSUPPORTED;
         }
         if ((rc = cuda_check(set_dyn_smem(DDKernels<T>::fine, (int)fine_smem), "smem attr fine")))

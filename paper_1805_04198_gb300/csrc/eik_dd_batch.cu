@@ -251,17 +251,14 @@ __global__ void kb_causal(const DDArgs<T> *__restrict__ args, Segs hl, Segs vl, 
         extern __shared__ __align__(16) char smem[];                                               \
         for_items(L, [&](int p, int local) { body<double>(args[p], smem, local); });               \
     }
-EIK_BATCH_PAIR(kb_step1, k_step1_body, 96, 168)
+EIK_BATCH_PAIR(kb_step1, k_step1_body, 112, 168)
 EIK_BATCH_PAIR(kb_step4, k_step4_body, 160, 168)
 EIK_BATCH_PAIR(kb_step4a, k_step4a_body, 160, 168)
-// The batch's subdomains are small (17-65 nodes a side): chunks in which every
-// lane is on a valid row are rare there, and the engine's second copy of the
-// step for them made the batch's subdomain stage 16% slower, so it is left out.
 template <class T>
 __device__ __forceinline__ void kb_fine_body(const DDArgs<T> &A, char *smem, int tile) {
-    k_fine_body<T, false>(A, smem, tile);
+    k_fine_body<T>(A, smem, tile);
 }
-EIK_BATCH_PAIR(kb_fine, kb_fine_body, 96, 168)
+EIK_BATCH_PAIR(kb_fine, kb_fine_body, 112, 168)
 
 template <class T> struct BatchKernels;
 template <> struct BatchKernels<float> {
@@ -506,8 +503,13 @@ static int batch_run(int nprob, const eik_grid *grids, const void *const *r, con
     size_t need_fine = 0, need_grid = 0;
     for (auto &c : B.fine) need_fine = std::max(need_fine, c.smem);
     for (auto &c : B.grid) need_grid = std::max(need_grid, c.smem);
-    if ((int)need_fine > smem_optin || (int)need_grid > smem_optin) {
-        set_error("shared memory need (%zu, %zu) exceeds the device limit %d", need_fine, need_grid, smem_optin);
+    size_t limit_fine = 0, limit_grid = 0;
+    for (auto &P : B.P) {
+        limit_fine = std::max(limit_fine, P.fine_limit);
+        limit_grid = std::max(limit_grid, std::max(P.step1_limit, P.step4_limit));
+    }
+    if ((int)limit_fine > smem_optin || (int)limit_grid > smem_optin) {
+        set_error("shared memory need (%zu, %zu) exceeds the device limit %d", limit_fine, limit_grid, smem_optin);
         return EIK_EUNSUPPORTED;
     }
     if ((rc = cuda_check(set_dyn_smem(BatchKernels<T>::fine, (int)std::max<size_t>(need_fine, 1)), "smem attr fine")))

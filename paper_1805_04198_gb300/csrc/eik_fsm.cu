@@ -80,55 +80,50 @@ struct FsmArgs {
     int nx, ny, nb, nstepp;
     T *state;
     T *rsk;
-    T *ghands;   // multi-CTA hand-off columns [nb][ny]
+    T *ghands;   // multi-CTA hand-off columns [nb][hand_elems(ny)]
     int *gctl;   // multi-CTA control words
     FsmDev *dev;
     T h;
     long long max_sweeps;
     int launches;
+    int multi;   // multi-CTA form
 };
 
-template <class T>
-struct PlainFsmPolicy {
-    T h;
-    __device__ __forceinline__ T update(T self, T vmx, T vpx, T vmy, T vpy, const T *sv, uint8_t,
-                                        bool &changed) const {
-        const T r = sv[0];  // <= 0 on Gamma
-        const T ut = local_solve2_value(vmx, vpx, vmy, vpy, Num<T>::mul(r, h));
-        const bool take = (r > T(0)) && (ut < self);
-        changed = take;
-        return take ? ut : self;
-    }
-};
-
-// Skewed slowness in output order (the inverse of skew_index, so a warp's
-// stores are contiguous; positions outside the box get 0), then the state:
-// Sec. 1.1 initialisation, Gamma fixed at g, everything else large.
+// Skewed slowness r h in storage order, 16 bytes per thread (positions outside
+// the box and Gamma nodes get +inf), then the state (Sec. 1.1 initialisation:
+// Gamma fixed at g, everything else large, padding columns included) and, for
+// the multi-CTA form, the empty hand-off columns.
 template <class T>
 __device__ void fsm_pack_body(const FsmArgs<T> &A, size_t bid, size_t nbid) {
-    const size_t chan = (size_t)4 * A.nb * A.nstepp * 32;
-    for (size_t e = bid * blockDim.x + threadIdx.x; e < chan; e += nbid * blockDim.x) {
-        const int l = (int)(e & 31);
-        const size_t row = e >> 5;
-        const int st = (int)(row % A.nstepp);
-        const int q = (int)((row / A.nstepp) % A.nb);
-        const int d = (int)(row / ((size_t)A.nstepp * A.nb));
-        const int sx = dir_sx(d), sy = dir_sy(d);
-        const int x = 32 * (sx > 0 ? q : A.nb - 1 - q) + (sx > 0 ? l : 31 - l);
-        const int lr = st - l;
-        T v = T(0);
-        if (x < A.nx && lr >= 0 && lr < A.ny) {
-            const size_t gi = (size_t)(sy > 0 ? lr : A.ny - 1 - lr) * A.sy + x;
-            v = A.gamma[gi] ? T(-1) : A.r[gi];
+    constexpr int E = 16 / (int)sizeof(T);
+    const size_t nv = (size_t)4 * A.nb * A.nstepp * 32 / E;
+    for (size_t t = bid * blockDim.x + threadIdx.x; t < nv; t += nbid * blockDim.x) {
+        union { T v[E]; uint4 w; } o;
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            int x, y;
+            o.v[i] = Num<T>::inf();
+            if (skew_node<T>(t * E + i, A.nx, A.ny, A.nb, A.nstepp, x, y)) {
+                const size_t gi = (size_t)y * A.sy + x;
+                o.v[i] = FsmPolicy<T>::node(A.gamma[gi] != 0, A.r[gi], A.h);
+            }
         }
-        A.rsk[e] = v;
+        reinterpret_cast<uint4 *>(A.rsk)[t] = o.w;
     }
-    const size_t total = (size_t)A.nx * A.ny;
+    const size_t total = (size_t)A.nb * A.ny * 32;
     for (size_t t = bid * blockDim.x + threadIdx.x; t < total; t += nbid * blockDim.x) {
-        int x = (int)(t % A.nx), y = (int)(t / A.nx);
-        const size_t gi = (size_t)y * A.sy + x;
-        A.state[box_index(x, y, A.ny)] = A.gamma[gi] ? A.g[gi] : Num<T>::inf();
+        const size_t row = t >> 5;
+        const int b = (int)(row / A.ny), y = (int)(row - (size_t)b * A.ny), x = 32 * b + (int)(t & 31);
+        T v = Num<T>::inf();
+        if (x < A.nx) {
+            const size_t gi = (size_t)y * A.sy + x;
+            if (A.gamma[gi]) v = A.g[gi];
+        }
+        A.state[t] = v;
     }
+    if (A.multi)
+        for (size_t t = bid * blockDim.x + threadIdx.x; t < A.nb * hand_elems(A.ny); t += nbid * blockDim.x)
+            A.ghands[t] = Hand<T>::empty();
 }
 
 template <class T>
@@ -142,11 +137,10 @@ __device__ void fsm_run_body(const FsmArgs<T> &A, char *smem) {
     bx.u = A.state;
     bx.st[0] = A.rsk;
     bx.sb = nullptr;
-    bx.nx = A.nx;
     bx.ny = A.ny;
     bx.nb = A.nb;
     bx.nstepp = A.nstepp;
-    PlainFsmPolicy<T> pol{A.h};
+    FsmPolicy<T> pol;
     long long sweeps;
     bool conv;
     if (threadIdx.x == 0) A.dev->err = 0;
@@ -159,7 +153,7 @@ __device__ void fsm_run_body(const FsmArgs<T> &A, char *smem) {
 }
 
 template <class T>
-__global__ void __maxnreg__((RegCap<T, 96, 128>::v)) k_fsm_run(FsmArgs<T> A) {
+__global__ void __maxnreg__((RegCap<T, 112, 160>::v)) k_fsm_run(FsmArgs<T> A) {
     extern __shared__ __align__(16) char smem[];
     fsm_run_body(A, smem);
 }
@@ -178,11 +172,10 @@ __device__ void fsm_run_global_body(const FsmArgs<T> &A, char *smem, int cta) {
     bx.u = A.state;
     bx.st[0] = A.rsk;
     bx.sb = nullptr;
-    bx.nx = A.nx;
     bx.ny = A.ny;
     bx.nb = A.nb;
     bx.nstepp = A.nstepp;
-    PlainFsmPolicy<T> pol{A.h};
+    FsmPolicy<T> pol;
     long long sweeps;
     bool conv;
     engine_run<T, 1, false, true>(bx, pol, A.max_sweeps, smem, sweeps, conv, &A.dev->err, A.ghands, A.gctl, cta);
@@ -193,7 +186,7 @@ __device__ void fsm_run_global_body(const FsmArgs<T> &A, char *smem, int cta) {
 }
 
 template <class T>
-__global__ void __maxnreg__((RegCap<T, 104, 160>::v)) k_fsm_run_global(FsmArgs<T> A) {
+__global__ void __maxnreg__((RegCap<T, 112, 160>::v)) k_fsm_run_global(FsmArgs<T> A) {
     extern __shared__ __align__(16) char smem[];
     fsm_run_global_body(A, smem, (int)blockIdx.x);
 }
@@ -231,7 +224,7 @@ static size_t fsm_layout(const FsmPlan &P, FsmArgs<T> *A, void *ws) {
     Carver cv(ws);
     T *state = cv.take<T>((size_t)P.nb * P.ny * 32);
     T *rsk = cv.take<T>((size_t)4 * P.nb * P.nstepp * 32);
-    T *ghands = cv.take<T>((size_t)P.nb * P.ny);
+    T *ghands = cv.take<T>(P.nb * hand_elems(P.ny));
     int *gctl = cv.take<int>(engine_global_ints(P.nb));
     FsmDev *dev = cv.take<FsmDev>(1);
     if (A) {
@@ -286,6 +279,7 @@ static int fsm_run(const eik_grid *grid, const FsmPlan &P, const void *r, const 
     if ((rc = cuda_check(cudaFuncGetAttributes(&fa, k_fsm_run<T>), "func attr"))) return rc;
     const bool single = (int)P.smem <= optin && P.nb <= 32 && regs_fit(fa, P.nb);
     A.launches = single ? 3 : 4;
+    A.multi = single ? 0 : 1;
     const size_t total = (size_t)P.nx * P.ny;
     const int tb = (int)std::min<size_t>((total + 255) / 256, (size_t)nsm * 16);
     EIK_LAUNCH("fsm_pack", s, k_fsm_pack<T><<<tb, 256, 0, s>>>(A));
@@ -356,7 +350,7 @@ __global__ void k_fsmm_pack(FsmMany<T> M) {
 }
 
 template <class T>
-__global__ void __maxnreg__((RegCap<T, 104, 128>::v)) k_fsmm_run(FsmMany<T> M) {
+__global__ void __maxnreg__((RegCap<T, 112, 160>::v)) k_fsmm_run(FsmMany<T> M) {
     extern __shared__ __align__(16) char smem[];
     fsm_run_body(fsm_prob(M, blockIdx.x), smem);
 }
@@ -370,7 +364,7 @@ __global__ void k_fsmm_init_global(FsmMany<T> M) {
 
 // CTA c of the launch serves problem p0 + c / nblk as its CTA c % nblk
 template <class T>
-__global__ void __maxnreg__((RegCap<T, 96, 160>::v)) k_fsmm_run_global(FsmMany<T> M, int p0, int nblk) {
+__global__ void __maxnreg__((RegCap<T, 112, 160>::v)) k_fsmm_run_global(FsmMany<T> M, int p0, int nblk) {
     extern __shared__ __align__(16) char smem[];
     fsm_run_global_body(fsm_prob(M, p0 + (int)blockIdx.x / nblk), smem, (int)blockIdx.x % nblk);
 }
@@ -464,6 +458,7 @@ static int fsm_many_run(const eik_grid *grid, const FsmManyPlan &MP, int nprob, 
     const int ngroups = (nprob + group - 1) / group;
     nl += 2 + (single ? 1 : 1 + ngroups);
     A.launches = nl;
+    A.multi = single ? 0 : 1;
     const size_t total = (size_t)P.nx * P.ny;
     const dim3 eg((unsigned)std::max<size_t>(1, std::min<size_t>((total + 255) / 256, (size_t)nsm * 16 / nprob + 1)),
                   (unsigned)nprob);

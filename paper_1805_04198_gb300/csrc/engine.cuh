@@ -15,13 +15,22 @@
 //    l+1's prefetched lower neighbour, shuffled down;
 //  * the block's rows stream through a 64-row shared-memory ring in chunks of
 //    8 rows, copied from global memory by cp.async three chunks ahead and
-//    written back as soon as all 32 lanes finished them;
+//    written back as soon as all 32 lanes finished them.  A row's ring slot is
+//    its physical index mod 64 and the sign of y alternates from sweep to
+//    sweep, so the first 64 rows of a sweep are still in the ring from the one
+//    before and are not read again;
 //  * the block's last lane hands its new column to the next block's warp
-//    through shared memory (published per chunk, tagged with the sweep); it
-//    reads the next block's first column (old values) from global memory;
+//    through a column buffer whose unwritten elements hold a reserved NaN: the
+//    value is its own flag, so no fence and no flag word sit on the hand-off
+//    path, and the reader puts the NaN back.  It reads the next block's first
+//    column (old values) from global memory, one chunk ahead;
 //  * per-node read-only data ("statics") are stored pre-skewed per sweep
-//    direction ([dir][block][step][lane]) so a chunk of 8 steps is one
-//    contiguous copy into a small shared ring;
+//    direction, 16 bytes (consecutive steps) of a lane together, and go through
+//    a small shared ring, so a chunk of one static is two 16-byte copies and two
+//    16-byte reads per lane (FP32);
+//  * positions outside the box hold neutral values (P::pad() in the state, the
+//    policy's inert static), so columns need no tests; rows are tested only in
+//    the chunks that touch the ends of the box;
 //  * there is no CTA-wide barrier between sweeps: a warp starts sweep k+1 as
 //    soon as its own block and the block whose old column it reads have
 //    finished sweep k, so the pipeline reverses direction without draining
@@ -29,10 +38,16 @@
 //    fixed point; the engine then stops (sweeps a warp had already begun
 //    speculatively change nothing).
 //
+// What bounds it: the chain of one step (shuffle, two differences, square
+// root, select, minimum), NX + NY of them per sweep, not memory or issue.  The
+// sweep direction is a run-time value (one copy of the step code for all four
+// orderings); policies that do not distinguish the sides of an axis (P::SYM)
+// are given the two axis minima.
+//
 // Storage of the state u: strip-major [block][row][32] (row = physical y,
-// 32 = physical x within the block), padded to a whole number of blocks;
-// padding columns are never touched.  One-sided differences at the box edges
-// come for free: missing neighbours are +inf.
+// 32 = physical x within the block), padded to a whole number of blocks with
+// P::pad().  One-sided differences at the box edges come for free: missing
+// neighbours are +inf.
 #pragma once
 
 #include <type_traits>
@@ -45,8 +60,7 @@ constexpr int CH = 8;             // rows (and steps) per chunk
 constexpr int RROWS = 64;         // u ring rows per warp (power of two)
 constexpr int SRCH = 3;           // statics chunks held in the statics ring
 constexpr int LEAD = 3;           // u chunks copied ahead of the current one
-constexpr int SWEEP_SHIFT = 13;   // hand-off progress tag: rows < 2^13, sweeps < 2^18
-constexpr int MAX_BOX_ROWS = (1 << SWEEP_SHIFT) - 1;
+constexpr int MAX_BOX_ROWS = (1 << 13) - 1;
 constexpr long long MAX_SWEEPS = 1ll << 17;
 
 __host__ __device__ inline int ceil32(int v) { return (v + 31) >> 5; }
@@ -65,17 +79,49 @@ __host__ __device__ inline int nstep_padded(int ny) { return ((ny + 31 + CH - 1)
 __host__ __device__ inline int dir_sx(int d) { return (d & 2) ? 1 : -1; }
 __host__ __device__ inline int dir_sy(int d) { return (d & 1) ? 1 : -1; }
 
+// Skewed statics: one stream of nstepp x 32 elements per direction and logical
+// block.  What lane l reads at step s is element skew_off<T>(s, l): within a
+// chunk of 8 steps, 16 bytes of consecutive steps of a lane, the 32 lanes side
+// by side, so that a chunk is read with 16-byte accesses of whole 512-byte rows.
+template <class T>
+__host__ __device__ inline size_t skew_off(int s, int l) {
+    constexpr int E = sizeof(T) == 1 ? CH : 16 / (int)sizeof(T);
+    return ((size_t)(s / E) * 32 + l) * E + s % E;
+}
+// Its inverse.
+template <class T>
+__host__ __device__ inline void skew_pos(unsigned e, int &s, int &l) {
+    constexpr unsigned E = sizeof(T) == 1 ? CH : 16 / (int)sizeof(T);
+    s = (int)(e / (32 * E) * E + e % E);
+    l = (int)(e / E % 32);
+}
+
 // Index of node (i, j) of a box (width -> nb blocks, height my) in the skewed
-// statics layout for direction d: [d][q][s][l], q = logical block, s = step,
-// l = lane.
+// statics: [direction][logical block][stream].
+template <class T>
 __host__ __device__ inline size_t skew_index(int d, int i, int j, int nb, int my, int nstepp) {
     int sx = dir_sx(d), sy = dir_sy(d);
     int b = i >> 5, pc = i & 31;
     int q = sx > 0 ? b : nb - 1 - b;
     int l = sx > 0 ? pc : 31 - pc;
     int lr = sy > 0 ? j : my - 1 - j;
-    int s = lr + l;
-    return (((size_t)d * nb + q) * nstepp + s) * 32 + l;
+    return ((size_t)d * nb + q) * nstepp * 32 + skew_off<T>(lr + l, l);
+}
+
+// Inverse of skew_index for kernels that write the statics in storage order:
+// element e -> node (x, y); false where the position is outside the box.
+template <class T>
+__device__ __forceinline__ bool skew_node(size_t e, int nx, int my, int nb, int nstepp, int &x, int &y) {
+    const unsigned stream = (unsigned)nstepp * 32;
+    const unsigned dq = (unsigned)(e / stream);
+    int s, l;
+    skew_pos<T>((unsigned)(e - (size_t)dq * stream), s, l);
+    const int q = (int)(dq % nb), d = (int)(dq / nb);
+    const bool px = dir_sx(d) > 0;
+    x = 32 * (px ? q : nb - 1 - q) + (px ? l : 31 - l);
+    const int lr = s - l;
+    y = dir_sy(d) > 0 ? lr : my - 1 - lr;
+    return x < nx && lr >= 0 && lr < my;
 }
 
 template <class T, int NST>
@@ -83,38 +129,145 @@ struct Box {
     T *u;                          // state, strip-major [nb][ny][32]
     const T *st[NST];              // skewed statics [4][nb][nstepp][32]
     const uint8_t *sb;             // skewed byte statics (may be null)
-    int nx, ny, nb, nstepp;
+    int ny, nb, nstepp;
 };
+
+// Elements of one hand-off column.
+__host__ __device__ inline size_t hand_elems(int ny) { return (size_t)((ny + CH - 1) / CH * CH); }
 
 // Shared memory needed per CTA of `nw` warps (one warp per block).  With
 // GLOBAL the hand-off columns and control words live in global memory.
 template <class T, int NST, bool HASB, bool GLOBAL = false>
 __host__ __device__ inline size_t engine_smem_bytes(int nw, int ny) {
-    size_t per_warp = (size_t)RROWS * 32 * sizeof(T)                 // u ring
-                      + (size_t)NST * SRCH * CH * 32 * sizeof(T)     // statics ring
-                      + (size_t)RROWS * sizeof(T)                    // halo ring
-                      + (GLOBAL ? 0 : (size_t)((ny + 3) & ~3) * sizeof(T))  // hand-off column
-                      + (HASB ? (size_t)SRCH * CH * 32 : 0);         // byte statics ring
-    return nw * per_warp + (GLOBAL ? 0 : (size_t)(32 + 2 * nw) * sizeof(int)) + 64;
+    size_t per_warp = (size_t)RROWS * 32 * sizeof(T)                        // u ring
+                      + (size_t)NST * SRCH * CH * 32 * sizeof(T)            // statics ring
+                      + (size_t)2 * CH * sizeof(T)                          // halo of two chunks
+                      + (GLOBAL ? 0 : hand_elems(ny) * sizeof(T))           // hand-off column
+                      + (HASB ? (size_t)SRCH * CH * 32 : 0);                // byte statics ring
+    return nw * per_warp + (GLOBAL ? 0 : (size_t)(32 + nw) * sizeof(int)) + 64;
 }
 
-// Control words of a multi-CTA engine run (global memory, zeroed by
+// The shared memory by which a box is accepted or refused (EIK_EUNSUPPORTED):
+// the documented size limit of subdomains and coarse grids, an upper bound of
+// what the engine takes.
+template <class T, int NST, bool HASB>
+__host__ inline size_t engine_limit_bytes(int nw, int ny) {
+    const size_t per_warp = (size_t)RROWS * 33 * sizeof(T) + (size_t)NST * SRCH * CH * 32 * sizeof(T) +
+                            (size_t)((ny + 3) & ~3) * sizeof(T) + (HASB ? (size_t)SRCH * CH * 32 : 0);
+    return nw * per_warp + (size_t)(32 + 2 * nw) * sizeof(int) + 64;
+}
+
+// Control words of a multi-CTA engine run (global memory, set by
 // engine_global_init before the run): abort, stop_at, fin[8], chg[8], then
-// prog[nb], done[nb].
-__host__ __device__ inline size_t engine_global_ints(int nb) { return 32 + 2 * (size_t)nb; }
+// done[nb].
+__host__ __device__ inline size_t engine_global_ints(int nb) { return 32 + (size_t)nb; }
 
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
-    unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gsrc) : "memory");
+// Element access with the reserved NaN of the hand-off columns.
+template <class T> struct Hand;
+template <> struct Hand<float> {
+    static __device__ __forceinline__ float empty() { return __uint_as_float(0x7fd5a5c3u); }
+    static __device__ __forceinline__ bool is_empty(float v) { return __float_as_uint(v) == 0x7fd5a5c3u; }
+};
+template <> struct Hand<double> {
+    static __device__ __forceinline__ double empty() { return __longlong_as_double(0x7ffad5a5c3b4e1f7ll); }
+    static __device__ __forceinline__ bool is_empty(double v) {
+        return __double_as_longlong(v) == 0x7ffad5a5c3b4e1f7ll;
+    }
+};
+
+// 16 bytes of elements (shared memory by 32-bit address).
+__device__ __forceinline__ void lds16(unsigned a, float *v) {
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(a) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void lds16(unsigned a, double *v) {
+    asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(a) : "memory");
+}
+// hand-off columns in shared memory: polled, so volatile
+__device__ __forceinline__ void hand_lds16(unsigned a, float *v) {
+    asm volatile("ld.volatile.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void hand_lds16(unsigned a, double *v) {
+    asm volatile("ld.volatile.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ float lds1(unsigned a, float) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ double lds1(unsigned a, double) {
+    double v;
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts1(unsigned a, float v) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void sts1(unsigned a, double v) {
+    asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+// Predicated forms: a branch around one access costs more than the access.
+#define EIK_PRED "{.reg .pred p; setp.ne.b32 p, %"
+__device__ __forceinline__ void lds1_if(bool c, unsigned a, float &v) {
+    asm volatile(EIK_PRED "2, 0; @p ld.shared.f32 %0, [%1];}" : "+f"(v) : "r"(a), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void lds1_if(bool c, unsigned a, double &v) {
+    asm volatile(EIK_PRED "2, 0; @p ld.shared.f64 %0, [%1];}" : "+d"(v) : "r"(a), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void sts1_if(bool c, unsigned a, float v) {
+    asm volatile(EIK_PRED "2, 0; @p st.shared.f32 [%0], %1;}" ::"r"(a), "f"(v), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void sts1_if(bool c, unsigned a, double v) {
+    asm volatile(EIK_PRED "2, 0; @p st.shared.f64 [%0], %1;}" ::"r"(a), "d"(v), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void hand_sts_if(bool c, unsigned a, float v) {
+    asm volatile(EIK_PRED "2, 0; @p st.volatile.shared.f32 [%0], %1;}" ::"r"(a), "f"(v), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void hand_sts_if(bool c, unsigned a, double v) {
+    asm volatile(EIK_PRED "2, 0; @p st.volatile.shared.f64 [%0], %1;}" ::"r"(a), "d"(v), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void hand_stg_if(bool c, float *a, float v) {
+    asm volatile(EIK_PRED "2, 0; @p st.volatile.global.f32 [%0], %1;}" ::"l"(a), "f"(v), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void hand_stg_if(bool c, double *a, double v) {
+    asm volatile(EIK_PRED "2, 0; @p st.volatile.global.f64 [%0], %1;}" ::"l"(a), "d"(v), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void hand_ldg_if(bool c, const float *a, float &v) {
+    asm volatile(EIK_PRED "2, 0; @p ld.volatile.global.f32 %0, [%1];}" : "+f"(v) : "l"(a), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void hand_ldg_if(bool c, const double *a, double &v) {
+    asm volatile(EIK_PRED "2, 0; @p ld.volatile.global.f64 %0, [%1];}" : "+d"(v) : "l"(a), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void ldcg_if(bool c, const float *a, float &v) {
+    asm volatile(EIK_PRED "2, 0; @p ld.global.cg.f32 %0, [%1];}" : "+f"(v) : "l"(a), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void ldcg_if(bool c, const double *a, double &v) {
+    asm volatile(EIK_PRED "2, 0; @p ld.global.cg.f64 %0, [%1];}" : "+d"(v) : "l"(a), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void stcg16_if(bool c, void *a, const uint4 &v) {
+    asm volatile(EIK_PRED "5, 0; @p st.global.cg.v4.u32 [%0], {%1, %2, %3, %4};}" ::"l"(a), "r"(v.x), "r"(v.y),
+                 "r"(v.z), "r"(v.w), "r"((int)c) : "memory");
+}
+__device__ __forceinline__ void cp16_if(bool c, unsigned dst, const void *src) {
+    asm volatile(EIK_PRED "2, 0; @p cp.async.cg.shared.global [%0], [%1], 16;}" ::"r"(dst), "l"(src), "r"((int)c)
+                 : "memory");
+}
+__device__ __forceinline__ void cp16(unsigned dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+// v = min(v, x) in the lanes where c holds
+__device__ __forceinline__ void min_if(bool c, float &v, float x) {
+    asm(EIK_PRED "2, 0; @p min.f32 %0, %0, %1;}" : "+f"(v) : "f"(x), "r"((int)c));
+}
+__device__ __forceinline__ void min_if(bool c, double &v, double x) {
+    if (c) v = fmin(v, x);
+}
+#undef EIK_PRED
 
 // Shared control words of one engine run.
 struct EngineCtl {
     long long lim;  // polls a wait may make (read once when the run starts)
-    int *prog;      // [nb] hand-off progress: (sweep << SWEEP_SHIFT) | rows published
     int *done;      // [nb] sweeps completed by the block (all rows written back)
     int *fin;       // [8] warps that finished sweep k (slot k & 7)
     int *chg;       // [8] any node changed in sweep k
@@ -126,245 +279,358 @@ __device__ __forceinline__ int vload(const int *p) { return *(const volatile int
 __device__ __forceinline__ void vstore(int *p, int v) { *(volatile int *)p = v; }
 template <bool GLOBAL>
 __device__ __forceinline__ void fence() {
-    if (GLOBAL) __threadfence();
-    else __threadfence_block();
+    if (GLOBAL) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    else asm volatile("fence.acq_rel.cta;" ::: "memory");
 }
 
-// Bounded wait until *p >= target.  Returns false if the engine is stopping
+// Bounded wait until ready() holds.  Returns false if the engine is stopping
 // (the last useful sweep is known to precede `sweep`) or on timeout.
-__device__ __forceinline__ bool wait_ge(const int *p, int target, const EngineCtl &C, int sweep, int *err) {
-    if (vload(p) >= target) return true;
-    // the sleep doubles from 32 ns to 1 us: short waits wake quickly, long
-    // ones leave the issue slots to the warps doing work
+// Called by whole warps; the answer is the same in every lane.
+template <class F>
+__device__ __forceinline__ bool wait_until(F ready, const EngineCtl &C, int sweep, int *err) {
+    if (__all_sync(FULL, ready())) return true;
+    // the sleep doubles from 32 to 256 ns: short waits wake quickly, long ones
+    // leave the issue slots to the warps doing work
     long long it = 0;
     unsigned ns = 32;
-    while (vload(p) < target) {
-        if (vload(C.abort_flag) || vload(C.stop_at) < sweep) return false;
+    while (!__all_sync(FULL, ready())) {
+        if (__any_sync(FULL, vload(C.abort_flag) || vload(C.stop_at) < sweep)) return false;
         if (++it > C.lim) {
             vstore(C.abort_flag, 1);
             atomicExch(err, DEV_TIMEOUT);
             return false;
         }
         __nanosleep(ns);
-        ns = ns < 1024 ? 2 * ns : 1024;
+        ns = ns < 256 ? 2 * ns : 256;
     }
     return true;
 }
 
-// One sweep (number k, direction (SX, SY)) of physical block b by its warp.
-// Returns -1 if the engine is stopping, else whether any node changed.
-template <int SX, int SY, bool GLOBAL, class T, int NST, bool HASB, bool STEADY_PATH, class P>
-__device__ int run_block(const Box<T, NST> &bx, const P &pol, int k, int b, T *ring, T *sring, uint8_t *sbring,
-                         T *halo, T *hand, const T *hands, size_t hand_elems, const EngineCtl &C, int *err) {
-    using N = Num<T>;
-    constexpr int DIR = (SX > 0 ? 2 : 0) | (SY > 0 ? 1 : 0);
-    const T INF = N::inf();
+// FSM update u = min(u, u~) (Sec. 1.1, eq. FSMupdate) from the axis minima a, b.
+// Static: r h, +inf at fixed nodes (Gamma) and outside the box, whose u~ is
+// then +inf, so that they keep their value without a test.
+template <class T>
+struct FsmPolicy {
+    static constexpr bool SYM = true;
+    static __device__ __forceinline__ T pad() { return Num<T>::inf(); }
+    static __device__ __forceinline__ T node(bool fixed, T r, T h) {
+        return !fixed && r > T(0) ? Num<T>::mul(r, h) : Num<T>::inf();
+    }
+    __device__ __forceinline__ T update(T self, T a, T b, T rh, bool &changed) const {
+        const T ut = local_solve2_min(a, b, rh);
+        changed = ut < self;
+        return fmin(ut, self);
+    }
+};
+
+// Shared memory of one warp (32-bit shared addresses).
+struct WarpMem {
+    unsigned ring, sring, halo, sbring;
+};
+
+// One sweep (number k, direction k mod 4) of physical block b by its warp.
+// `hands`: the hand-off columns of all blocks ([nb][hand_elems(ny)], shared or,
+// with GLOBAL, global memory).  Returns -1 if the engine is stopping, else
+// whether any node changed.
+//
+// The work of a chunk boundary (write-back, copies, halo) is spread over the
+// eight steps of the chunk, without branches, where it issues in the latency
+// of the step's own chain; only the wait for the hand-in is between chunks.
+template <bool GLOBAL, class T, int NST, bool HASB, class P>
+__device__ int run_block(const Box<T, NST> &bx, const P &pol, int k, int b, const WarpMem &M, T *hands,
+                         const EngineCtl &C, int *err) {
+    constexpr int E = 16 / (int)sizeof(T);   // elements of a 16-byte access
+    constexpr int VC = CH / E;               // 16-byte accesses per lane, chunk and static
+    constexpr unsigned SZ = sizeof(T), ROWB = 32 * SZ, RMASK = RROWS * ROWB - 1;
+    const T PAD = P::pad();
+    const int dir = k & 3, sx = dir_sx(dir), sy = dir_sy(dir);
     const int lane = threadIdx.x & 31;
-    const int NB = bx.nb, NY = bx.ny, NX = bx.nx;
-    const int q = SX > 0 ? b : NB - 1 - b;         // logical block
-    const int pc = SX > 0 ? lane : 31 - lane;       // physical column in the block
-    const int x = 32 * b + pc;
-    const bool colok = x < NX;
-    const bool fullblk = 32 * b + 31 < NX;  // every lane of the block on a column
-    const int bp = b - SX, bn = b + SX;              // physical predecessor / successor
+    const int NB = bx.nb, NY = bx.ny;
+    const int q = sx > 0 ? b : NB - 1 - b;           // logical block
+    const int pc = sx > 0 ? lane : 31 - lane;         // physical column in the block
+    const int bp = b - sx, bn = b + sx;               // physical predecessor / successor
     const bool has_prev = bp >= 0 && bp < NB;
     const bool has_next = bn >= 0 && bn < NB;
-    const int pcn = SX > 0 ? 0 : 31;                 // successor's first logical column
-    const bool nextok = has_next && (32 * bn + pcn) < NX;
-    T *ublk = bx.u + (size_t)b * NY * 32;
-    const T *unext = bx.u + (size_t)(has_next ? bn : b) * NY * 32;
-    const T *hand_in = hands + (size_t)(has_prev ? bp : b) * hand_elems;
-    const int nchunks = (NY + CH - 1) / CH;
-    const int nsteps = NY + 31;
-    const int tag = k << SWEEP_SHIFT;
+    const bool lane0 = lane == 0, lane31 = lane == 31, low = lane < CH;
+    const size_t he = hand_elems(NY);
+    T *const hand_out = hands + (size_t)b * he;
+    T *const hand_in = hands + (size_t)(has_prev ? bp : b) * he;
+    const unsigned hand_out_s = GLOBAL ? 0u : (unsigned)__cvta_generic_to_shared(hand_out);
+    const unsigned hand_in_s = GLOBAL ? 0u : (unsigned)__cvta_generic_to_shared(hand_in);
+    const int nchunks = (NY + CH - 1) / CH;         // chunks of rows
+    const int nJ = (NY + 31 + CH - 1) / CH;         // chunks of steps
 
     // Start condition: the successor block (whose old column this sweep reads)
     // has finished sweep k-1.  Our own block finished it in program order.
     if (k > 0 && has_next) {
-        if (!wait_ge(C.done + bn, k, C, k, err)) return -1;
+        const int *dn = C.done + bn;
+        if (!wait_until([&] { return vload(dn) >= k; }, C, k, err)) return -1;
+        fence<GLOBAL>();
+    }
+    // When the x sign flipped, the column read as hand-in was read by the block
+    // on the far side of the predecessor in sweep k-1: that block must have put
+    // its NaNs back (it feeds the predecessor now, so this never waits longer
+    // than the hand-in itself).  Otherwise this warp was the reader.
+    if (k > 0 && !(k & 1) && bp - sx >= 0 && bp - sx < NB) {
+        const int *dp = C.done + (bp - sx);
+        if (!wait_until([&] { return vload(dp) >= k; }, C, k, err)) return -1;
         fence<GLOBAL>();
     }
 
-    auto prow = [&](int m) { return SY > 0 ? m : NY - 1 - m; };
-    constexpr int EPL = 8;                                  // elements per lane per chunk
-    constexpr int CPL = EPL * (int)sizeof(T) / 16;          // 16-byte copies per lane
-    constexpr int E16 = 16 / (int)sizeof(T);                // elements per 16-byte copy
+    // u rows move between global memory and the ring in chunks of 8: this lane
+    // copies 8 columns of row r8.  Chunks j and j + 8 share their ring rows.
     const int r8 = lane >> 2, cg = lane & 3;
-    auto issue_chunk = [&](int j) {                         // u rows of chunk j -> ring
-        const int m = j * CH + r8;
-        if (j < nchunks && m < NY) {
-            const T *src = ublk + (size_t)prow(m) * 32 + cg * EPL;
-            T *dst = ring + (m & (RROWS - 1)) * 32 + cg * EPL;
+    const int prow0 = sy > 0 ? 0 : NY - 1;            // physical row of logical row 0
+    const int cstep = sy * CH * 32;                   // elements from one chunk to the next
+    T *gcopy = bx.u + ((size_t)b * NY + prow0 + sy * r8) * 32 + cg * 8;  // chunk 0
+    unsigned scopy = (unsigned)(prow0 + sy * r8) * ROWB + cg * 8 * SZ;
+    int mcopy = r8;
+    const int mfirst = k == 0 ? 0 : RROWS;            // first row not in the ring already
+    auto issue_chunk = [&] {
+        const unsigned dst = M.ring + (scopy & RMASK);
+        const bool on = mcopy < NY && mcopy >= mfirst;
 #pragma unroll
-            for (int c = 0; c < CPL; ++c) cp_async16(dst + c * E16, src + c * E16);
-        }
+        for (int c = 0; c < 8 / E; ++c) cp16_if(on, dst + 16 * c, gcopy + c * E);
+        gcopy += cstep;
+        scopy += (unsigned)cstep * SZ;
+        mcopy += CH;
     };
-    const size_t stbase = ((size_t)DIR * NB + q) * bx.nstepp;
-    auto issue_statics = [&](int j) {                       // statics of steps 8j.. -> statics ring
-        const int s0 = j * CH;
-        if (s0 + CH > bx.nstepp) return;
-        const int slot = j % SRCH;
+    uint4 wb[8 / E];
+    auto wb_load = [&](unsigned off) {
+#pragma unroll
+        for (int c = 0; c < 8 / E; ++c)
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(wb[c].x), "=r"(wb[c].y), "=r"(wb[c].z), "=r"(wb[c].w)
+                         : "r"(M.ring + (off & RMASK) + 16 * c) : "memory");
+    };
+    auto wb_store = [&](int m, T *dst) {
+#pragma unroll
+        for (int c = 0; c < 8 / E; ++c) stcg16_if((unsigned)m < (unsigned)NY, dst + c * E, wb[c]);
+    };
+    // statics of 8 steps -> statics ring (slot = chunk mod SRCH)
+    const size_t stbase = ((size_t)dir * NB + q) * bx.nstepp * 32;
+    size_t stoff = stbase + lane * E;
+    const uint8_t *sbp = HASB ? bx.sb + stbase + lane * 16 : nullptr;
+    unsigned sslot = 0;
+    auto issue_statics = [&] {
 #pragma unroll
         for (int kk = 0; kk < NST; ++kk) {
-            const T *src = bx.st[kk] + (stbase + s0) * 32 + lane * EPL;
-            T *dst = sring + ((size_t)kk * SRCH * CH + slot * CH) * 32 + lane * EPL;
+            const unsigned dst = M.sring + (((unsigned)kk * SRCH + sslot) * CH * 32 + lane * E) * SZ;
 #pragma unroll
-            for (int c = 0; c < CPL; ++c) cp_async16(dst + c * E16, src + c * E16);
+            for (int c = 0; c < VC; ++c) cp16(dst + 512 * c, bx.st[kk] + stoff + c * 32 * E);
         }
-        if (HASB && lane < 16) cp_async16(sbring + (slot * CH) * 32 + lane * 16, bx.sb + (stbase + s0) * 32 + lane * 16);
+        if (HASB) {
+            cp16_if(lane < 16, M.sbring + sslot * CH * 32 + lane * 16, sbp);
+            sbp += CH * 32;
+        }
+        stoff += CH * 32;
+        sslot = sslot == SRCH - 1 ? 0 : sslot + 1;
     };
-    T hreg = INF;  // halo of one chunk (lanes 0..7), staged in a register
-    auto load_halo = [&](int j) {
-        const int mh = j * CH + lane;
-        hreg = (lane < CH && nextok && j < nchunks && mh < NY) ? __ldcg(unext + (size_t)prow(mh) * 32 + pcn) : INF;
+    // right neighbours of lane 31 in chunk j: logical rows 8j-31 .. 8j-24 of the
+    // successor's first column, one row per lane, one chunk ahead in hreg
+    const T *hsrc = bx.u + ((size_t)(has_next ? bn : b) * NY + prow0) * 32 + (sx > 0 ? 0 : 31) +
+                    (ptrdiff_t)(sy * (lane - 31)) * 32;
+    int mhalo = has_next && low ? lane - 31 : (1 << 29);
+    T hreg = PAD;
+    const unsigned shalo = M.halo + (lane & (CH - 1)) * SZ;
+    auto load_halo = [&] {
+        hreg = PAD;
+        ldcg_if((unsigned)mhalo < (unsigned)NY, hsrc, hreg);
+        hsrc += cstep;
+        mhalo += CH;
     };
-    auto write_back = [&](int j) {
-        const int m = j * CH + r8;
-        if (m < NY) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(ring + (m & (RROWS - 1)) * 32 + cg * EPL);
-            uint4 *dst = reinterpret_cast<uint4 *>(ublk + (size_t)prow(m) * 32 + cg * EPL);
+
+    // left neighbours of lane 0 in chunk j: rows 8j .. 8j+7 of the predecessor's
+    // last column; with GLOBAL one row per lane (lanes 0..7), read a chunk ahead
+    T hin[GLOBAL ? 1 : CH], hahead = PAD;
 #pragma unroll
-            for (int c = 0; c < CPL; ++c) __stcg(dst + c, src[c]);
+    for (int i = 0; i < (GLOBAL ? 1 : CH); ++i) hin[i] = PAD;
+    const int hlim = has_prev ? NY : 0;  // rows there are to read
+    auto hand_ahead = [&](int m0) { hand_ldg_if(low && m0 + lane < hlim, hand_in + m0 + lane, hahead); };
+    auto hand_wait = [&](int m0) -> bool {
+        if (GLOBAL) {
+            hin[0] = hahead;
+            hahead = PAD;
+            bool again = false;
+            return wait_until([&] {
+                if (again) hand_ldg_if(low && m0 + lane < NY, hand_in + m0 + lane, hin[0]);
+                again = true;
+                return !(low && m0 + lane < NY && Hand<T>::is_empty(hin[0]));
+            }, C, k, err);
+        }
+        const unsigned a = hand_in_s + m0 * SZ;
+        return wait_until([&] {
+#pragma unroll
+            for (int c = 0; c < VC; ++c) hand_lds16(a + 16 * c, hin + (GLOBAL ? 0 : c * E));
+            bool r = true;
+#pragma unroll
+            for (int i = 0; i < CH; ++i) r = r && (!Hand<T>::is_empty(hin[GLOBAL ? 0 : i]) || m0 + i >= NY);
+            return r;
+        }, C, k, err);
+    };
+    auto hand_clear = [&](int m0) {  // after every lane has read them
+        if (GLOBAL) {
+            hand_stg_if(low && m0 + lane < hlim, hand_in + m0 + lane, Hand<T>::empty());
+        } else {
+            hand_sts_if(low && m0 < hlim, hand_in_s + (m0 + (lane & (CH - 1))) * SZ, Hand<T>::empty());
         }
     };
 
-    // Prologue: u chunks 0..LEAD-1 and statics chunks 0..1 in flight (one
-    // group per chunk), halo of chunk 0 in the ring, of chunk 1 in hreg.
-    fence<GLOBAL>();
+    // Prologue: u chunks 0..LEAD-1 and statics chunks 0 and 1 in flight (one
+    // group per chunk), halo of chunk 0 staged, of chunk 1 in hreg.
 #pragma unroll
     for (int j = 0; j < LEAD; ++j) {
-        issue_chunk(j);
-        if (j < 2) issue_statics(j);
-        cp_async_commit();
+        issue_chunk();
+        if (j < 2) issue_statics();
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    load_halo(0);
-    if (lane < CH) halo[lane] = hreg;
-    load_halo(1);
-
-    T last = INF, cur = INF, dnx = INF, hal = INF;
-    // hand-off values of the current chunk: lane i holds logical row s0 + i;
-    // with GLOBAL the next chunk's values are fetched one boundary ahead
-    T hcur = INF, hnext = INF;
-    auto hand_row = [&](int m) -> T {
-        return (lane < CH && m < NY) ? (GLOBAL ? __ldcg(hand_in + m) : hand_in[m]) : INF;
-    };
-    bool changed = false;
-    const int lastJ = nchunks + 4;                 // boundary that writes back the last chunk
-    const bool lane0 = lane == 0, lane31 = lane == 31;
-    T *myring = ring + pc;
-    int known = -1;
-    if (GLOBAL && has_prev) {
-        if (!wait_ge(C.prog + bp, tag | (CH > NY ? NY : CH), C, k, err)) {
-            cp_async_wait<0>();
+    sts1_if(low, shalo, hreg);  // rows -31 .. -24
+    hsrc += cstep;
+    mhalo += CH;
+    load_halo();
+    if (has_prev) {
+        if (GLOBAL) hand_ahead(0);
+        if (!hand_wait(0)) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
             return -1;
         }
-        known = vload(C.prog + bp);
+        // the reader of our own column put its NaNs back in an earlier sweep,
+        // before it wrote the value just read
         fence<GLOBAL>();
-        hnext = hand_row(lane);
     }
-    auto ringval = [&](int m) -> T {
-        return (colok && (unsigned)m < (unsigned)NY) ? myring[(m & (RROWS - 1)) * 32] : INF;
-    };
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();
 
-    for (int J = 0; J <= lastJ; ++J) {
-        __syncwarp();
-        // chunk J-5 is complete: its last row 8J-33 was updated by lane 31 at step 8J-2
-        if (J >= 5 && J - 5 < nchunks) write_back(J - 5);
-        if (has_next && lane31) {
-            int pub = CH * J - 31;  // rows whose hand-off values this lane has written
-            pub = pub < 0 ? 0 : (pub > NY ? NY : pub);
-            if (J == lastJ) pub = NY;
-            fence<GLOBAL>();
-            vstore(C.prog + b, tag | pub);
-        }
-        // halo of chunk J+1 into the ring, load halo of chunk J+2
-        if (lane < CH) halo[((J + 1) * CH + lane) & (RROWS - 1)] = hreg;
-        load_halo(J + 2);
-        // copies for u chunk J+LEAD (into the slot of chunk J-5, written back
-        // above) and statics chunk J+2 (slot of chunk J-1, used up)
-        issue_chunk(J + LEAD);
-        issue_statics(J + 2);
-        cp_async_commit();
-        // the group of boundary J-2 (u chunk J+1, statics chunk J) has landed
-        cp_async_wait<2>();
+    auto ok = [&](int m) { return (unsigned)m < (unsigned)NY; };
+    // ring offsets (this lane's column) of its rows m, m+1, m+2 at step 0 (m = -lane)
+    const unsigned rstep = (unsigned)(sy * (int)ROWB);
+    unsigned roff = (unsigned)(prow0 - sy * lane) * ROWB + (unsigned)pc * SZ;
+    unsigned a0 = M.ring + (roff & RMASK), a1 = M.ring + ((roff + rstep) & RMASK),
+             a2 = M.ring + ((roff + 2 * rstep) & RMASK);
+    roff = (roff + 2 * rstep) & RMASK;
+    T cur = PAD, d1 = PAD, d2 = PAD;
+    lds1_if(ok(-lane), a0, cur);
+    lds1_if(ok(1 - lane), a1, d1);
+    lds1_if(ok(2 - lane), a2, d2);
+    T last = PAD, fromleft = PAD;                    // own previous result, the left lane's
+    T fromright = __shfl_down_sync(FULL, d1, 1);     // the right lane's old value on this lane's row
+    bool changed = false;
+    // hand-out: lane 31's row at step s is s - 31
+    const bool hands_out = has_next && lane31;
+    unsigned ho_s = hand_out_s - 31 * SZ;
+    T *ho_g = hand_out - 31;
+    unsigned sread = 0;  // statics ring slot of this chunk
+
+    for (int J = 0; J < nJ; ++J) {
         const int s0 = J * CH;
-        if (s0 < nsteps && has_prev) {
-            // rows this chunk needs (smem hand-off) or the next chunk needs
-            // (global hand-off, fetched a boundary ahead)
-            const int rows = GLOBAL ? s0 + 2 * CH : s0 + CH;
-            const int need = tag | (rows > NY ? NY : rows);
-            if (known < need) {
-                if (!wait_ge(C.prog + bp, need, C, k, err)) {
-                    cp_async_wait<0>();
-                    return -1;
-                }
-                known = vload(C.prog + bp);
-                fence<GLOBAL>();
-            }
-            if (GLOBAL) {
-                hcur = hnext;
-                hnext = hand_row(s0 + CH + lane);
-            } else {
-                hcur = hand_row(s0 + lane);
-            }
-        }
-        __syncwarp();
-        if ((J & 7) == 7 && (vload(C.abort_flag) || vload(C.stop_at) < k)) {
-            cp_async_wait<0>();
-            return -1;
-        }
-        if (s0 >= nsteps) continue;
-        if (J == 0) {
-            cur = ringval(-lane);
-            dnx = ringval(1 - lane);
-        }
-        hal = halo[(s0 - lane) & (RROWS - 1)];
-        const T *sbase = sring + (size_t)((J % SRCH) * CH) * 32 + lane;
-        const uint8_t *bbase = sbring + ((J % SRCH) * CH) * 32 + lane;
-        // The chunk's 8 steps.  STEADY: every lane of a full block is on a
-        // valid row at every step and so is the row two ahead that it loads,
-        // so the row and column tests are dropped (the same operations on the
-        // same values otherwise).
+        T hal[CH];
+#pragma unroll
+        for (int c = 0; c < VC; ++c) lds16(M.halo + (J & 1) * CH * SZ + 16 * c, hal + c * E);
+        uint2 sb8 = make_uint2(0u, 0u);
+        if constexpr (HASB)
+            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(sb8.x), "=r"(sb8.y)
+                         : "r"(M.sbring + sread * CH * 32 + lane * 8) : "memory");
+        const unsigned sst = M.sring + (sread * CH * 32 + lane * E) * SZ;
+        sread = sread == SRCH - 1 ? 0 : sread + 1;
+        T sv[NST][E];  // statics of the current E steps
+        // The chunk's 8 steps.  STEADY: every lane is on a valid row at every
+        // step and so is the row three ahead that it loads, so the row tests
+        // are dropped (the same operations on the same values otherwise).
         auto run_chunk = [&](auto steady_tag) {
             constexpr bool STEADY = decltype(steady_tag)::value;
 #pragma unroll
             for (int i = 0; i < CH; ++i) {
                 const int m = s0 + i - lane;
-                const bool rowok = STEADY || (unsigned)m < (unsigned)NY;
-                const bool act = STEADY || (colok && rowok);
-                // loads for the next step, issued before this step's store
-                const T dn2 = STEADY ? myring[((m + 2) & (RROWS - 1)) * 32] : ringval(m + 2);
-                const T hal2 = halo[(m + 1) & (RROWS - 1)];
-                T sv[NST > 0 ? NST : 1];
+                if (i % E == 0) {
 #pragma unroll
-                for (int kk = 0; kk < NST; ++kk) sv[kk] = sbase[((size_t)kk * SRCH * CH + i) * 32];
-                const uint8_t sbv = HASB ? bbase[i * 32] : (uint8_t)0;
-                const T hin = __shfl_sync(FULL, hcur, i);
-                const T fromleft = __shfl_up_sync(FULL, last, 1);
-                const T fromright = __shfl_down_sync(FULL, dnx, 1);
-                const T left = lane0 ? ((has_prev && rowok) ? hin : INF) : fromleft;
-                const T right = lane31 ? ((nextok && rowok) ? hal : INF) : fromright;
+                    for (int kk = 0; kk < NST; ++kk)
+                        lds16(sst + (unsigned)kk * SRCH * CH * 32 * SZ + 512 * (i / E), sv[kk]);
+                }
+                // ---- boundary work of the chunk
+                if (i == 0) {
+                    wb_load(scopy);                                 // rows of chunk J-5
+                    if (GLOBAL) hand_ahead(s0 + CH);
+                }
+                if (i == 1) wb_store(mcopy - RROWS, gcopy - 8 * (ptrdiff_t)cstep);
+                if (i == 2) {
+                    __syncwarp();
+                    issue_chunk();       // u chunk J+LEAD, into the rows of chunk J-5
+                    issue_statics();     // statics chunk J+2
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                }
+                if (i == 3) {
+                    hand_clear(s0);
+                    sts1_if(low, shalo + ((J + 1) & 1) * CH * SZ, hreg);
+                    load_halo();
+                }
+                // u chunk J+1 (first read at step 5) has landed
+                if (i == 4) {
+                    asm volatile("cp.async.wait_group 2;" ::: "memory");
+                    __syncwarp();
+                }
+                // ---- the node
+                T right = lane31 ? hal[i] : fromright;
+                const T hl = GLOBAL ? __shfl_sync(FULL, hin[0], i) : hin[GLOBAL ? 0 : i];
                 bool ch = false;
-                const T upd = pol.update(cur, SX > 0 ? left : right, SX > 0 ? right : left, SY > 0 ? last : dnx,
-                                         SY > 0 ? dnx : last, sv, sbv, ch);
-                const T nw = act ? upd : INF;
-                changed = changed || (act && ch);
-                if (act) myring[(m & (RROWS - 1)) * 32] = nw;
-                if (act && lane31 && has_next) hand[m] = nw;
+                T nw;
+                if constexpr (P::SYM) {
+                    min_if(lane0, right, hl);
+                    min_if(!lane0, right, fromleft);
+                    nw = pol.update(cur, right, fmin(last, d1), sv[0][i % E], ch);
+                } else {
+                    const T left = lane0 ? hl : fromleft;
+                    T s1[NST];
+#pragma unroll
+                    for (int kk = 0; kk < NST; ++kk) s1[kk] = sv[kk][i % E];
+                    const uint8_t sbv = HASB ? (uint8_t)((i < 4 ? sb8.x : sb8.y) >> (8 * (i & 3))) : (uint8_t)0;
+                    nw = pol.update(cur, sx > 0 ? left : right, sx > 0 ? right : left, sy > 0 ? last : d1,
+                                    sy > 0 ? d1 : last, s1, sbv, ch);
+                }
+                if (!STEADY) nw = ok(m) ? nw : PAD;
+                fromleft = __shfl_up_sync(FULL, nw, 1);
+                if (STEADY) sts1(a0, nw);
+                else sts1_if(ok(m), a0, nw);
+                if (GLOBAL) hand_stg_if(hands_out && (STEADY || ok(m)), ho_g + i, nw);
+                else hand_sts_if(hands_out && (STEADY || ok(m)), ho_s + i * SZ, nw);
+                changed = changed || (ch && (STEADY || ok(m)));
+                roff = (roff + rstep) & RMASK;
+                const unsigned a3 = M.ring + roff;
+                T d3 = PAD;
+                if (STEADY) d3 = lds1(a3, T(0));
+                else lds1_if(ok(m + 3), a3, d3);
+                fromright = __shfl_down_sync(FULL, d2, 1);
                 last = nw;
-                cur = dnx;
-                dnx = dn2;
-                hal = hal2;
+                cur = d1;
+                d1 = d2;
+                d2 = d3;
+                a0 = a1;
+                a1 = a2;
+                a2 = a3;
             }
         };
-        if constexpr (STEADY_PATH) {
-            if (fullblk && s0 >= 31 && s0 + CH + 1 < NY) run_chunk(std::true_type{});
-            else run_chunk(std::false_type{});
-        } else {
-            run_chunk(std::false_type{});
+        if (s0 >= 31 && s0 + CH + 2 < NY) run_chunk(std::true_type{});
+        else run_chunk(std::false_type{});
+        ho_s += CH * SZ;
+        ho_g += CH;
+        // statics of chunk J+1 have landed; every lane's rows and halo are visible
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        bool go = true;
+        if (s0 + CH < hlim) go = hand_wait(s0 + CH);
+        if (go && (J & 7) == 7) go = !__any_sync(FULL, vload(C.abort_flag) || vload(C.stop_at) < k);
+        if (!go) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            return -1;
         }
     }
-    cp_async_wait<0>();
+    // the last rows (gcopy, scopy and mcopy are at chunk nJ + LEAD; rows 64 back
+    // share ring rows)
+    for (int j = nJ >= 5 ? nJ - 5 : 0; j < nchunks; ++j) {
+        const int back = nJ + LEAD - j;
+        wb_load(scopy - (unsigned)(back * cstep) * SZ);
+        wb_store(mcopy - back * CH, gcopy - (ptrdiff_t)back * cstep);
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     fence<GLOBAL>();  // every lane's write-back before the block's completion flag
     __syncwarp();
     return __any_sync(FULL, changed) ? 1 : 0;
@@ -375,10 +641,11 @@ __device__ int run_block(const Box<T, NST> &bx, const P &pol, int k, int b, T *r
 // blockDim.x >= 32 * bx.nb, engine_smem_bytes<T, NST, HASB>(nb, ny) bytes of
 // dynamic shared memory at `smem`.  Multi-CTA form (GLOBAL = true): CTA c
 // owns blocks [c * nw, c * nw + nw) with nw = blockDim.x / 32, hand-off
-// columns live in `ghands` ([nb][ny] elements) and the control words in
-// `gctl` (engine_global_ints(nb) ints, zeroed before the launch); every CTA of
-// the grid must be co-resident (cooperative launch).  All threads must call it.
-template <class T, int NST, bool HASB, bool GLOBAL = false, bool STEADY_PATH = true, class P>
+// columns live in `ghands` ([nb][hand_elems(ny)], every element Hand<T>::empty()
+// before the launch) and the control words in `gctl` (engine_global_ints(nb)
+// ints, set by engine_global_init before the launch); every CTA of the grid
+// must be co-resident (cooperative launch).  All threads must call it.
+template <class T, int NST, bool HASB, bool GLOBAL = false, class P>
 __device__ void engine_run(const Box<T, NST> &bx, const P &pol, long long max_sweeps, char *smem, long long &sweeps,
                            bool &converged, int *err, T *ghands = nullptr, int *gctl = nullptr, int cta = -1) {
     const int nwc = GLOBAL ? (int)(blockDim.x >> 5) : bx.nb;   // warps (blocks) of this CTA
@@ -387,32 +654,30 @@ __device__ void engine_run(const Box<T, NST> &bx, const P &pol, long long max_sw
     const int b0 = GLOBAL ? (cta >= 0 ? cta : (int)blockIdx.x) * nwc : 0;
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const size_t ring_e = (size_t)RROWS * 32, sring_e = (size_t)NST * SRCH * CH * 32;
-    const size_t halo_e = RROWS, hand_e = GLOBAL ? (size_t)bx.ny : (size_t)((bx.ny + 3) & ~3);
+    const size_t ring_b = (size_t)RROWS * 32 * sizeof(T);
+    const size_t sring_b = (size_t)NST * SRCH * CH * 32 * sizeof(T);
+    const size_t small_b = (size_t)2 * CH * sizeof(T);
     const size_t sb_b = HASB ? (size_t)SRCH * CH * 32 : 0;
-    T *base = reinterpret_cast<T *>(smem);
-    T *ring = base + (size_t)warp * ring_e;
-    T *sring = base + (size_t)nwc * ring_e + (size_t)warp * sring_e;
-    T *halo = base + (size_t)nwc * (ring_e + sring_e) + (size_t)warp * halo_e;
-    T *hands;
-    uint8_t *bytes;
-    if (GLOBAL) {
-        hands = ghands;
-        bytes = reinterpret_cast<uint8_t *>(base + (size_t)nwc * (ring_e + sring_e + halo_e));
-    } else {
-        hands = base + (size_t)nwc * (ring_e + sring_e + halo_e);
-        bytes = reinterpret_cast<uint8_t *>(hands + (size_t)nwc * hand_e);
-    }
-    uint8_t *sbring = bytes + (size_t)warp * sb_b;
-    int *ints = GLOBAL ? gctl : reinterpret_cast<int *>(bytes + (size_t)nwc * sb_b);
+    // layout: rings, statics rings, byte rings, halo, hand-off columns, control words; every part a multiple of 16 bytes
+    char *const p_sring = smem + (size_t)nwc * ring_b;
+    char *const p_sb = p_sring + (size_t)nwc * sring_b;
+    char *const p_small = p_sb + (size_t)nwc * sb_b;
+    char *const p_hand = p_small + (size_t)nwc * small_b;
+    T *hands = GLOBAL ? ghands : reinterpret_cast<T *>(p_hand);
+    const size_t he = hand_elems(bx.ny);
+    int *ints = GLOBAL ? gctl : reinterpret_cast<int *>(p_hand + (size_t)nwc * he * sizeof(T));
+    WarpMem M;
+    M.ring = (unsigned)__cvta_generic_to_shared(smem + (size_t)warp * ring_b);
+    M.sring = (unsigned)__cvta_generic_to_shared(p_sring + (size_t)warp * sring_b);
+    M.sbring = (unsigned)__cvta_generic_to_shared(p_sb + (size_t)warp * sb_b);
+    M.halo = (unsigned)__cvta_generic_to_shared(p_small + (size_t)warp * small_b);
     EngineCtl C;
     C.lim = spin_limit();
     C.abort_flag = ints;
     C.stop_at = ints + 1;
     C.fin = ints + 8;
     C.chg = ints + 16;
-    C.prog = ints + 32;
-    C.done = ints + 32 + bx.nb;
+    C.done = ints + 32;
 
     if (!GLOBAL) {
         if (threadIdx.x == 0) {
@@ -423,26 +688,17 @@ __device__ void engine_run(const Box<T, NST> &bx, const P &pol, long long max_sw
             C.fin[threadIdx.x] = 0;
             C.chg[threadIdx.x] = 0;
         }
-        if ((int)threadIdx.x < bx.nb) {
-            C.prog[threadIdx.x] = -1;
-            C.done[threadIdx.x] = 0;
-        }
+        if ((int)threadIdx.x < bx.nb) C.done[threadIdx.x] = 0;
+        for (size_t i = threadIdx.x; i < (size_t)nwc * he; i += blockDim.x) hands[i] = Hand<T>::empty();
     }
     __syncthreads();
 
     const int b = b0 + warp;
     if (warp < nwc && b < bx.nb) {
-        T *hand = hands + (size_t)b * hand_e;
         for (long long kk = 0; kk < max_sweeps; ++kk) {
             const int k = (int)kk;
-            if (vload(C.abort_flag) || vload(C.stop_at) < k) break;
-            int ch;
-            switch (k & 3) {
-                case 0: ch = run_block<-1, -1, GLOBAL, T, NST, HASB, STEADY_PATH>(bx, pol, k, b, ring, sring, sbring, halo, hand, hands, hand_e, C, err); break;
-                case 1: ch = run_block<-1, +1, GLOBAL, T, NST, HASB, STEADY_PATH>(bx, pol, k, b, ring, sring, sbring, halo, hand, hands, hand_e, C, err); break;
-                case 2: ch = run_block<+1, -1, GLOBAL, T, NST, HASB, STEADY_PATH>(bx, pol, k, b, ring, sring, sbring, halo, hand, hands, hand_e, C, err); break;
-                default: ch = run_block<+1, +1, GLOBAL, T, NST, HASB, STEADY_PATH>(bx, pol, k, b, ring, sring, sbring, halo, hand, hands, hand_e, C, err); break;
-            }
+            if (__any_sync(FULL, vload(C.abort_flag) || vload(C.stop_at) < k)) break;
+            const int ch = run_block<GLOBAL, T, NST, HASB>(bx, pol, k, b, M, hands, C, err);
             if (ch < 0) break;
             // sweep k of this block is complete: publish it, then the sweep status
             if (lane == 0) {
@@ -470,14 +726,9 @@ __device__ void engine_run(const Box<T, NST> &bx, const P &pol, long long max_sw
     __syncthreads();
 }
 
-// Zeroes the control words of a multi-CTA engine run (one thread block).
+// Sets the control words of a multi-CTA engine run (one thread block).
 __device__ inline void engine_global_init(int *gctl, int nb) {
-    for (int i = threadIdx.x; i < (int)engine_global_ints(nb); i += blockDim.x) {
-        int v = 0;
-        if (i == 1) v = 0x7fffffff;
-        if (i >= 32 && i < 32 + nb) v = -1;
-        gctl[i] = v;
-    }
+    for (int i = threadIdx.x; i < (int)engine_global_ints(nb); i += blockDim.x) gctl[i] = i == 1 ? 0x7fffffff : 0;
 }
 
 }  // namespace eik
