@@ -17,7 +17,85 @@ constexpr unsigned FULL = 0xffffffffu;
 
 template <class T> struct Num;
 
+// Comparisons of FP64 values on the integer pipe.  The FP64 pipe of this GPU
+// issues a warp instruction every 19 cycles per SM with 64 cycles of latency,
+// and a double comparison or minimum costs 100 to 157 cycles there; the
+// integer forms take about 25.  key() orders all non-NaN doubles as signed
+// integers (-0 just below +0); mag() is the order of magnitudes, in which a
+// NaN exceeds everything.
+// The bits go through asm: the compiler turns an integer comparison of bit-cast
+// doubles back into a floating-point one, which is slow and wrong for NaNs.
+__device__ __forceinline__ long long bits64(double a) {
+    long long x;
+    asm("mov.b64 %0, %1;" : "=l"(x) : "d"(a));
+    return x;
+}
+__device__ __forceinline__ long long key(double a) {
+    const long long x = bits64(a);
+    return x ^ ((x >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ long long mag(double a) { return bits64(a) & 0x7fffffffffffffffll; }
+
+// Correctly rounded square root of a normal x with exponent in [-900, 900]
+// (other values take the library root).  With x = 4^q m, m in [1, 4): an FP32
+// reciprocal root and one FP32 correction give g, the root of m to 2^-43, as a
+// multiple of 2^-43; the residual m - g^2 (at most 46 bits) is exact in one FP64
+// FMA; its leading 24 bits times y / 2 give the rest of the root to 2^-12 of an
+// ulp in fixed point.  Where that is within 2^-9.6 ulp of a rounding boundary
+// (one root in 400) the exact residual of the result decides (Markstein, "IA-64
+// and Elementary Functions", ch. 9): R = m - G^2 is a multiple of ulp^2, and G
+// is the rounded root unless R > G ulp or R <= -G ulp (R < 0 where G is a power
+// of two).  One operation on the FP64 pipe instead of about twenty dependent
+// ones.
+__device__ __forceinline__ double sqrt_rn64(double x) {
+    const int hi = __double2hiint(x);
+    const int lo = __double2loint(x);
+    const int e = (hi >> 20) - 1023;  // x > 0
+    const int par = e & 1, qe = (e - par) << 19;  // q in exponent position
+    const int mexp = par << 20;
+    const double m = __hiloint2double((hi & 0xfffff) | (mexp + (1023 << 20)), lo);
+    // m = mh + ml in FP32: 24 bits, the next 23
+    const float mh = __int_as_float((__funnelshift_l(lo, hi, 3) & 0x7fffff) | ((mexp << 3) + (127 << 23)));
+    const int mlx = (mexp << 3) + (104 << 23);
+    const float ml = __fsub_rn(__int_as_float(mlx | (int)((unsigned)(lo << 3) >> 9)), __int_as_float(mlx));
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(mh));
+    // in [1, 2), so that its FP64 ulp is 2^-52
+    const float s = fminf(fmaxf(__fmul_rn(mh, y), 1.f), 1.99999988f);
+    const float yh = __fmul_rn(0.5f, y);
+    const float c = __fmul_rn(__fadd_rn(__fmaf_rn(-s, s, mh), ml), yh);
+    // g = s + c, c in units of 2^-43 added to the bits of (double)s
+    const int ci = __float_as_int(__fmaf_rn(c, 8796093022208.f, 12582912.f)) - 0x4b400000;
+    const int sb = __float_as_int(s);
+    const long long gb = (((long long)((sb >> 3) + (896 << 20)) << 32) | (unsigned)(sb << 29)) + ((long long)ci << 9);
+    const double g = __longlong_as_double(gb);
+    const double r = __fma_rn(-g, g, m);
+    // r as FP32 (its leading bits, 2^-86 <= |r| <= 2^-40 or 0), the correction in 2^-11 ulp
+    const int rh = __double2hiint(r), rl = __double2loint(r);
+    const int rb = ((__funnelshift_l(rl, rh, 3) & 0x7fffffff) | (rh & 0x80000000)) - 0x40000000;
+    const float rf = (rh & 0x7fffffff) == 0 ? 0.f : __int_as_float(rb);
+    // + 1023: rounds to the nearest ulp by a shift
+    const int f = __float_as_int(__fmaf_rn(__fmul_rn(rf, yh), 9223372036854775808.f, 12582912.f)) - (0x4b400000 - 1023);
+    long long out = gb + (f >> 11);
+    if (((f + 3) & 2047) <= 4 || (unsigned)(e + 900) > 1800u) {
+        if ((unsigned)(e + 900) > 1800u) return __dsqrt_rn(x);
+        const double G = __longlong_as_double(out);
+        const long long Rb = bits64(__fma_rn(-G, G, m));
+        const long long ub = out - (52ll << 52);  // G * ulp(G), G in [1, 2)
+        const bool neg = Rb < 0;
+        const long long Rm = Rb & 0x7fffffffffffffffll;
+        // (G = 2, just above the largest root, stands at its lower neighbour's ulp)
+        const bool off = (neg ? Rm >= ub : Rm > ub) || (neg && (out & 0xfffffffffffffll) == 0 && Rm > 0);
+        if (off) out += neg ? -1 : 1;
+    }
+    return __longlong_as_double(out + ((long long)qe << 32));
+}
+
 template <> struct Num<float> {
+    static __device__ __forceinline__ bool lt(float a, float b) { return a < b; }
+    static __device__ __forceinline__ bool le(float a, float b) { return a <= b; }
+    static __device__ __forceinline__ float mn(float a, float b) { return fminf(a, b); }
+    static __device__ __forceinline__ bool below(float d, float rh) { return fabsf(d) < rh; }
     static __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
     static __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
     static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
@@ -36,13 +114,19 @@ template <> struct Num<float> {
 };
 
 template <> struct Num<double> {
+    // (operands are never NaN)
+    static __device__ __forceinline__ bool lt(double a, double b) { return key(a) < key(b); }
+    static __device__ __forceinline__ bool le(double a, double b) { return key(a) <= key(b); }
+    static __device__ __forceinline__ double mn(double a, double b) { return lt(a, b) ? a : b; }
+    // |d| < rh for rh >= 0, false where d is NaN
+    static __device__ __forceinline__ bool below(double d, double rh) { return mag(d) < bits64(rh); }
     static __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
     static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
     static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
     static __device__ __forceinline__ double sqrt_(double a) { return __dsqrt_rn(a); }
     static __device__ __forceinline__ double div(double a, double b) { return __ddiv_rn(a, b); }
     static __device__ __forceinline__ double inf() { return __longlong_as_double(0x7ff0000000000000ll); }
-    static __device__ __forceinline__ double sqrt_solve(double a) { return __dsqrt_rn(a); }
+    static __device__ __forceinline__ double sqrt_solve(double a) { return sqrt_rn64(a); }
 };
 
 // Wind packing: component a in {-1,0,+1} stored as (w+1) in 2 bits at 2a.
@@ -58,6 +142,42 @@ constexpr uint8_t WIND_ZERO = 0x15;  // (0,0,0)
 // echoes boundary data rather than a fine solution.
 constexpr uint8_t WIND_ECHO = 0x80;
 
+// Value of the local solve from the axis minima a, b: the two-term branch
+// (a + b + sqrt(2 r^2 h^2 - (a-b)^2)) / 2 where |a - b| < r h, else the smaller
+// one plus r h.  The discriminant needs no clamp: where the two-term branch is
+// taken it is at least (r h)^2; where it is negative or NaN its root is not
+// selected.
+__device__ __forceinline__ float solve2(float a, float b, float rh, bool &two) {
+    using N = Num<float>;
+    const float d = N::sub(a, b);
+    const float disc = N::sub(N::mul(N::mul(2.f, rh), rh), N::mul(d, d));
+    // (a + b + root) / 2 as one rounding of root / 2 + (a + b) / 2: halving is
+    // exact, so this is the same value with a shorter chain behind the root
+    const float u2 = __fmaf_rn(N::sqrt_solve(disc), 0.5f, N::mul(N::add(a, b), 0.5f));
+    const float u1 = N::add(fminf(a, b), rh);
+    two = fabsf(d) < rh;
+    return two ? u2 : u1;
+}
+// FP64: eight operations on the FP64 pipe, the comparisons, the doubling and the
+// halving on the integer pipe.  r h = +inf (fixed nodes) takes the one-term
+// branch, which gives +inf too.
+__device__ __forceinline__ double solve2(double a, double b, double rh, bool &two) {
+    using N = Num<double>;
+    const double d = N::sub(a, b);
+    two = N::below(d, rh) && __double2hiint(rh) < 0x7ff00000;
+    // 2 r h by its exponent (exact; where r h is subnormal its square is 0 in any case)
+    const double rh2 = __hiloint2double(__double2hiint(rh) + (1 << 20), __double2loint(rh));
+    const double disc = N::sub(N::mul(rh2, rh), N::mul(d, d));
+    const double w = N::add(N::add(a, b), sqrt_rn64(two ? disc : 1.0));
+    // w / 2 by its exponent, where that is exact (it always is but next to the
+    // ends of the FP64 range)
+    const int wh = __double2hiint(w);
+    double u2 = __hiloint2double(wh - (1 << 20), __double2loint(w));
+    if (two && ((unsigned)(wh & 0x7fffffff) - (2u << 20)) >= ((0x7ffu - 2u) << 20)) u2 = N::mul(w, 0.5);
+    const double u1 = N::add(N::mn(a, b), rh);
+    return two ? u2 : u1;
+}
+
 // 2-D Godunov local solve.  vm*/vp* are the neighbours on the minus/plus side
 // of each axis (+inf where missing: the one-sided rule of Sec. 1.1).  Returns
 // u~ and the packed wind of the branch taken (zero wind when u~ is +inf).
@@ -68,49 +188,26 @@ template <class T>
 __device__ __forceinline__ T local_solve2(T vmx, T vpx, T vmy, T vpy, T rh, uint8_t &wind) {
     using N = Num<T>;
     // Alg. 3: the smaller neighbour per axis; a tie goes to the plus side.
-    const bool lx = vmx < vpx, ly = vmy < vpy;
+    const bool lx = N::lt(vmx, vpx), ly = N::lt(vmy, vpy);
     const T a = lx ? vmx : vpx, b = ly ? vmy : vpy;
     const int sa = lx ? 1 : -1, sb = ly ? 1 : -1;
-    const T d = N::sub(a, b);
-    // two-term branch: (a + b + sqrt(2 r^2 h^2 - (a-b)^2)) / 2
-    const T disc = N::sub(N::mul(N::mul(T(2), rh), rh), N::mul(d, d));
-    const T u2 = N::mul(N::add(N::add(a, b), N::sqrt_solve(fmax(disc, T(0)))), T(0.5));
-    const bool two = fabs(d) < rh;
-    const bool ax = a < b;
-    const T u1 = N::add(ax ? a : b, rh);
-    const T u = two ? u2 : u1;
-    wind = two ? wind_pack(sa, sb) : (u < N::inf() ? (ax ? wind_pack(sa, 0) : wind_pack(0, sb)) : WIND_ZERO);
+    bool two;
+    const T u = solve2(a, b, rh, two);
+    wind = two ? wind_pack(sa, sb)
+               : (N::lt(u, N::inf()) ? (N::lt(a, b) ? wind_pack(sa, 0) : wind_pack(0, sb)) : WIND_ZERO);
     return u;
 }
 
 // Value-only variant used inside the sweeps (the wind is recomputed from the
-// converged state, so the sweeps need only the value), from the axis minima.
-// The two-term branch needs no clamp of the discriminant: where it is taken,
-// |a - b| < r h, the discriminant is at least (r h)^2; where it is negative or
-// NaN its root is not selected.  In FP64 the root of an unselected
-// discriminant is kept off the square root's slow path.
-__device__ __forceinline__ float local_solve2_min(float a, float b, float rh) {
-    using N = Num<float>;
-    const float d = N::sub(a, b);
-    const float disc = N::sub(N::mul(N::mul(2.f, rh), rh), N::mul(d, d));
-    // (a + b + root) / 2 as one rounding of root / 2 + (a + b) / 2: halving is
-    // exact, so this is the same value with a shorter chain behind the root
-    const float u2 = __fmaf_rn(N::sqrt_solve(disc), 0.5f, N::mul(N::add(a, b), 0.5f));
-    const float u1 = N::add(fmin(a, b), rh);
-    return fabsf(d) < rh ? u2 : u1;
-}
-__device__ __forceinline__ double local_solve2_min(double a, double b, double rh) {
-    using N = Num<double>;
-    const double d = N::sub(a, b);
-    const bool two = fabs(d) < rh;
-    const double disc = N::sub(N::mul(N::mul(2.0, rh), rh), N::mul(d, d));
-    const double u2 = N::mul(N::add(N::add(a, b), N::sqrt_solve(two ? disc : 1.0)), 0.5);
-    const double u1 = N::add(fmin(a, b), rh);
-    return two ? u2 : u1;
+// converged state, so the sweeps need only the value).
+template <class T>
+__device__ __forceinline__ T local_solve2_min(T a, T b, T rh) {
+    bool two;
+    return solve2(a, b, rh, two);
 }
 template <class T>
 __device__ __forceinline__ T local_solve2_value(T vmx, T vpx, T vmy, T vpy, T rh) {
-    return local_solve2_min(fmin(vmx, vpx), fmin(vmy, vpy), rh);
+    return local_solve2_min(Num<T>::mn(vmx, vpx), Num<T>::mn(vmy, vpy), rh);
 }
 
 // 3-D Godunov local solve: axis minima sorted a_p0 <= a_p1 <= a_p2 (ties keep
@@ -124,12 +221,13 @@ __device__ __forceinline__ T local_solve2_value(T vmx, T vpx, T vmy, T vpy, T rh
 template <class T>
 __device__ __forceinline__ T local_solve3(const T *vm, const T *vp, T rh, uint8_t &wind) {
     using N = Num<T>;
-    const bool l0 = vm[0] < vp[0], l1 = vm[1] < vp[1], l2 = vm[2] < vp[2];
+    const bool l0 = N::lt(vm[0], vp[0]), l1 = N::lt(vm[1], vp[1]), l2 = N::lt(vm[2], vp[2]);
     const T a0 = l0 ? vm[0] : vp[0], a1 = l1 ? vm[1] : vp[1], a2 = l2 ? vm[2] : vp[2];
     // stable ranks: axis b precedes axis c when a_b < a_c, or a_b == a_c and b < c
-    const int r0 = (a1 < a0 ? 1 : 0) + (a2 < a0 ? 1 : 0);
-    const int r1 = (a0 <= a1 ? 1 : 0) + (a2 < a1 ? 1 : 0);
-    const int r2 = (a0 <= a2 ? 1 : 0) + (a1 <= a2 ? 1 : 0);
+    const bool b10 = N::lt(a1, a0), b20 = N::lt(a2, a0), b21 = N::lt(a2, a1);
+    const int r0 = (b10 ? 1 : 0) + (b20 ? 1 : 0);
+    const int r1 = (b10 ? 0 : 1) + (b21 ? 1 : 0);
+    const int r2 = (b20 ? 0 : 1) + (b21 ? 0 : 1);
     const T v0 = r0 == 0 ? a0 : (r1 == 0 ? a1 : a2);
     const T v1 = r0 == 1 ? a0 : (r1 == 1 ? a1 : a2);
     const T v2 = r0 == 2 ? a0 : (r1 == 2 ? a1 : a2);

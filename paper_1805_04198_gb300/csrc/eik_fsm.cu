@@ -212,6 +212,12 @@ __global__ void k_fsm_unpack(FsmArgs<T> A, eik_fsm_stats *out) {
     fsm_unpack_body(A, out, blockIdx.x, gridDim.x);
 }
 
+// Widest grid (32-column blocks) swept by one CTA.  Above it the blocks' warps
+// share too few schedulers and spreading them over CTAs wins in spite of the
+// slower hand-off (FP32 us a sweep, one CTA / several: 257^2 50.6 / 51.2,
+// 513^2 114 / 97; FP64 129^2 171 / 179, 257^2 335 / 324).
+constexpr int MAX_SINGLE_NB = 9;
+
 struct FsmPlan {
     int nx, ny, nb, nstepp;
     size_t smem, bytes;
@@ -245,7 +251,9 @@ static bool fsm_plan(const eik_grid *grid, FsmPlan &P) {
     P.nstepp = nstep_padded(P.ny);
     P.smem = grid->dtype == EIK_F64 ? engine_smem_bytes<double, 1, false>(P.nb, P.ny)
                                      : engine_smem_bytes<float, 1, false>(P.nb, P.ny);
-    P.wpc = 2;
+    // FP64: one warp per CTA, each with an SM's FP64 pipe of its own (two warps
+    // share it: 1401 x 701 FP64 1119 us a sweep, one 1073); FP32: 1 to 4 are alike
+    P.wpc = grid->dtype == EIK_F64 ? 1 : 2;
     P.gsmem = grid->dtype == EIK_F64 ? engine_smem_bytes<double, 1, false, true>(P.wpc, P.ny)
                                       : engine_smem_bytes<float, 1, false, true>(P.wpc, P.ny);
     P.bytes = grid->dtype == EIK_F64 ? fsm_layout<double>(P, nullptr, nullptr) : fsm_layout<float>(P, nullptr, nullptr);
@@ -277,7 +285,7 @@ static int fsm_run(const eik_grid *grid, const FsmPlan &P, const void *r, const 
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     cudaFuncAttributes fa;
     if ((rc = cuda_check(cudaFuncGetAttributes(&fa, k_fsm_run<T>), "func attr"))) return rc;
-    const bool single = (int)P.smem <= optin && P.nb <= 32 && regs_fit(fa, P.nb);
+    const bool single = (int)P.smem <= optin && P.nb <= MAX_SINGLE_NB && regs_fit(fa, P.nb);
     A.launches = single ? 3 : 4;
     A.multi = single ? 0 : 1;
     const size_t total = (size_t)P.nx * P.ny;

@@ -261,7 +261,7 @@ __device__ __forceinline__ void min_if(bool c, float &v, float x) {
     asm(EIK_PRED "2, 0; @p min.f32 %0, %0, %1;}" : "+f"(v) : "f"(x), "r"((int)c));
 }
 __device__ __forceinline__ void min_if(bool c, double &v, double x) {
-    if (c) v = fmin(v, x);
+    if (c) v = Num<double>::mn(v, x);
 }
 #undef EIK_PRED
 
@@ -318,8 +318,8 @@ struct FsmPolicy {
     }
     __device__ __forceinline__ T update(T self, T a, T b, T rh, bool &changed) const {
         const T ut = local_solve2_min(a, b, rh);
-        changed = ut < self;
-        return fmin(ut, self);
+        changed = Num<T>::lt(ut, self);
+        return changed ? ut : self;
     }
 };
 
@@ -576,7 +576,7 @@ __device__ int run_block(const Box<T, NST> &bx, const P &pol, int k, int b, cons
                 if constexpr (P::SYM) {
                     min_if(lane0, right, hl);
                     min_if(!lane0, right, fromleft);
-                    nw = pol.update(cur, right, fmin(last, d1), sv[0][i % E], ch);
+                    nw = pol.update(cur, right, Num<T>::mn(last, d1), sv[0][i % E], ch);
                 } else {
                     const T left = lane0 ? hl : fromleft;
                     T s1[NST];
