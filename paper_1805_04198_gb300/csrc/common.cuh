@@ -150,7 +150,9 @@ constexpr uint8_t WIND_ECHO = 0x80;
 __device__ __forceinline__ float solve2(float a, float b, float rh, bool &two) {
     using N = Num<float>;
     const float d = N::sub(a, b);
-    const float disc = N::sub(N::mul(N::mul(2.f, rh), rh), N::mul(d, d));
+    // rn(2 r h r h) = 2 rn(r h r h): one product, and the doubling in the FMA (for
+    // r h below 2^-63, 1e-19, the product is subnormal and its root flushed to 0)
+    const float disc = __fmaf_rn(2.f, N::mul(rh, rh), -N::mul(d, d));
     // (a + b + root) / 2 as one rounding of root / 2 + (a + b) / 2: halving is
     // exact, so this is the same value with a shorter chain behind the root
     const float u2 = __fmaf_rn(N::sqrt_solve(disc), 0.5f, N::mul(N::add(a, b), 0.5f));
@@ -165,7 +167,8 @@ __device__ __forceinline__ double solve2(double a, double b, double rh, bool &tw
     using N = Num<double>;
     const double d = N::sub(a, b);
     two = N::below(d, rh) && __double2hiint(rh) < 0x7ff00000;
-    // 2 r h by its exponent (exact; where r h is subnormal its square is 0 in any case)
+    // 2 r h by its exponent (exact; where r h is subnormal its square is 0 in any
+    // case).  Not 2 (r h)^2: that loses the bits of a square just below the normal range.
     const double rh2 = __hiloint2double(__double2hiint(rh) + (1 << 20), __double2loint(rh));
     const double disc = N::sub(N::mul(rh2, rh), N::mul(d, d));
     const double w = N::add(N::add(a, b), sqrt_rn64(two ? disc : 1.0));
@@ -248,6 +251,60 @@ __device__ __forceinline__ T local_solve3(const T *vm, const T *vp, T rh, uint8_
     }
     const int nt = three ? 3 : (two ? 2 : (u < N::inf() ? 1 : 0));  // axes used, by rank
     wind = wind_pack(r0 < nt ? (l0 ? 1 : -1) : 0, r1 < nt ? (l1 ? 1 : -1) : 0, r2 < nt ? (l2 ? 1 : -1) : 0);
+    return u;
+}
+
+// x / 3, correctly rounded: the quotient by the rounded reciprocal corrected by
+// its exact residual (Markstein, as above; equal to the division for every
+// finite float but -0).  NaN at +-inf.
+__device__ __forceinline__ float div3(float x) {
+    const float c = 1.f / 3.f;
+    const float q = __fmul_rn(x, c);
+    return __fmaf_rn(__fmaf_rn(-3.f, q, x), c, q);
+}
+__device__ __forceinline__ double div3(double x) {
+    const double c = 1.0 / 3.0;
+    const double q = __dmul_rn(x, c);
+    return __fma_rn(__fma_rn(-3.0, q, x), c, q);
+}
+
+// Value of the 3-D local solve from the three axis minima (the same rounded
+// operations as local_solve3 on the sorted values): a sort of minima and maxima,
+// no winds.  r h = +inf (fixed nodes) gives +inf or, in FP32, NaN: neither is
+// below any value.
+__device__ __forceinline__ float solve3(float m0, float m1, float m2, float rh) {
+    using N = Num<float>;
+    const float lo = fminf(m0, m1), hi = fmaxf(m0, m1);
+    const float v0 = fminf(lo, m2), t = fmaxf(lo, m2);
+    const float v1 = fminf(t, hi), v2 = fmaxf(t, hi);
+    const float d1 = N::sub(v1, v0), d2 = N::sub(v2, v0);
+    const float dd = N::mul(d1, d1), rr = N::mul(rh, rh);
+    const float disc = __fmaf_rn(2.f, rr, -dd);
+    const float u2 = __fmaf_rn(N::sqrt_solve(disc), 0.5f, N::mul(N::add(v0, v1), 0.5f));
+    const bool two = d1 < rh;
+    const float sd = N::add(d1, d2);
+    const float disc3 = N::sub(N::mul(sd, sd), N::mul(3.f, N::sub(N::add(dd, N::mul(d2, d2)), rr)));
+    const float u3 = N::add(v0, div3(N::add(sd, N::sqrt_solve(fmaxf(disc3, 0.f)))));
+    const float u = two ? u2 : N::add(v0, rh);
+    return two && u2 > v2 ? u3 : u;
+}
+__device__ __forceinline__ double solve3(double m0, double m1, double m2, double rh) {
+    using N = Num<double>;
+    const bool s01 = N::lt(m1, m0);
+    const double lo = s01 ? m1 : m0, hi = s01 ? m0 : m1;
+    const bool s2 = N::lt(m2, lo);
+    const double v0 = s2 ? m2 : lo, t = s2 ? lo : m2;
+    const bool s3 = N::lt(t, hi);
+    const double v1 = s3 ? t : hi, v2 = s3 ? hi : t;
+    bool two;
+    double u = solve2(v0, v1, rh, two);
+    if (two && N::lt(v2, u)) {
+        const double d1 = N::sub(v1, v0), d2 = N::sub(v2, v0);
+        const double sd = N::add(d1, d2);
+        double disc3 = N::sub(N::mul(sd, sd), N::mul(3.0, N::sub(N::add(N::mul(d1, d1), N::mul(d2, d2)), N::mul(rh, rh))));
+        if (disc3 < 0.0) disc3 = 0.0;
+        u = N::add(v0, div3(N::add(sd, disc3 > 0.0 ? sqrt_rn64(disc3) : 0.0)));
+    }
     return u;
 }
 
