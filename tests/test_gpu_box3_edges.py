@@ -1,0 +1,47 @@
+"""3-D sweeps at the sizes where their schedules change, FP64 bitwise against the oracle: the tile form of the
+plain sweeping (8 x 4 column tiles, chunks of 4 steps) and the hyperplane form that larger grids take, and the
+subdomain boxes of the decomposition: partial tiles, more tiles than the warps hold, thin boxes without a border."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _problem(shape, seed, g0=0.0):
+    rng = np.random.default_rng(seed)
+    r = rng.uniform(0.5, 2.0, shape)
+    gamma = np.zeros(shape, np.uint8)
+    for _ in range(3):
+        gamma[tuple(rng.integers(0, s) for s in shape)] = 1
+    return r, gamma, g0 + rng.uniform(0.0, 0.1, shape)
+
+
+def _dev(*arrs):
+    return [torch.from_numpy(np.ascontiguousarray(a)).to(DEV) for a in arrs]
+
+
+@pytest.mark.parametrize("shape", [(2, 2, 2), (3, 4, 8), (4, 5, 9), (5, 3, 7), (8, 13, 17), (13, 8, 33), (29, 21, 16),
+                                   (40, 9, 25), (3, 430, 420)])
+def test_fsm3(gpu, shape):
+    r, gamma, g = _problem(shape, sum(shape), g0=-1.0 if shape[0] == 5 else 0.0)
+    u_ref, sweeps, _ = O.fsm(r, gamma, g, 0.05)
+    u, st = gpu.fsm(*_dev(r, gamma, g), 0.05)
+    np.testing.assert_array_equal(u.cpu().numpy(), u_ref)
+    assert st["sweeps"] == sweeps and st["converged"] == 1
+
+
+# tiles and cells per subdomain (x, y, z), coarse ratio
+@pytest.mark.parametrize("tiles,cells,c", [((2, 2, 2), (4, 4, 4), 4), ((2, 1, 2), (8, 8, 8), 4), ((1, 2, 2), (10, 6, 4), 2),
+                                           ((1, 1, 2), (64, 40, 4), 4), ((1, 1, 1), (2, 2, 2400), 2)])
+def test_dd3_boxes(gpu, tiles, cells, c):
+    shape = tuple(t * s + 1 for t, s in zip(reversed(tiles), reversed(cells)))
+    r, gamma, g = _problem(shape, 17 + sum(shape))
+    kw = dict(theta=0.2, max_iter=2, tol=0.0, max_coarse_sweeps=8)
+    u_ref, s_ref, _ = O.dd(r, gamma, g, 0.05, tiles, c, **kw)
+    u, st = gpu.dd_solve(*_dev(r, gamma, g), 0.05, tiles, c, **kw)
+    assert st["iters"] == s_ref["iters"]
+    np.testing.assert_array_equal(u.cpu().numpy(), u_ref)
