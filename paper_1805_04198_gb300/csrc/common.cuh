@@ -41,19 +41,30 @@ __device__ __forceinline__ long long mag(double a) { return bits64(a) & 0x7fffff
 // reciprocal root and one FP32 correction give g, the root of m to 2^-43, as a
 // multiple of 2^-43; the residual m - g^2 (at most 46 bits) is exact in one FP64
 // FMA; its leading 24 bits times y / 2 give the rest of the root to 2^-12 of an
-// ulp in fixed point.  Where that is within 2^-9.6 ulp of a rounding boundary
-// (one root in 400) the exact residual of the result decides (Markstein, "IA-64
+// ulp in fixed point.  Where that is within 2^-10.7 ulp of a rounding boundary
+// (one root in 800) the exact residual of the result decides (Markstein, "IA-64
 // and Elementary Functions", ch. 9): R = m - G^2 is a multiple of ulp^2, and G
 // is the rounded root unless R > G ulp or R <= -G ulp (R < 0 where G is a power
 // of two).  One operation on the FP64 pipe instead of about twenty dependent
-// ones.
-__device__ __forceinline__ double sqrt_rn64(double x) {
+// ones.  In two parts, so that several roots can be under way before the rare
+// second part splits the warp.
+struct Root64 {
+    double x, m;
+    long long out;  // bits of G
+    int qe;         // 2^q for the exponent field
+    bool unsure;
+    __device__ __forceinline__ double value() const { return __longlong_as_double(out + ((long long)qe << 32)); }
+};
+__device__ __forceinline__ Root64 root_start(double x) {
+    Root64 R;
+    R.x = x;
     const int hi = __double2hiint(x);
     const int lo = __double2loint(x);
     const int e = (hi >> 20) - 1023;  // x > 0
-    const int par = e & 1, qe = (e - par) << 19;  // q in exponent position
+    const int par = e & 1;
+    R.qe = (e - par) << 19;
     const int mexp = par << 20;
-    const double m = __hiloint2double((hi & 0xfffff) | (mexp + (1023 << 20)), lo);
+    R.m = __hiloint2double((hi & 0xfffff) | (mexp + (1023 << 20)), lo);
     // m = mh + ml in FP32: 24 bits, the next 23
     const float mh = __int_as_float((__funnelshift_l(lo, hi, 3) & 0x7fffff) | ((mexp << 3) + (127 << 23)));
     const int mlx = (mexp << 3) + (104 << 23);
@@ -69,26 +80,36 @@ __device__ __forceinline__ double sqrt_rn64(double x) {
     const int sb = __float_as_int(s);
     const long long gb = (((long long)((sb >> 3) + (896 << 20)) << 32) | (unsigned)(sb << 29)) + ((long long)ci << 9);
     const double g = __longlong_as_double(gb);
-    const double r = __fma_rn(-g, g, m);
-    // r as FP32 (its leading bits, 2^-86 <= |r| <= 2^-40 or 0), the correction in 2^-11 ulp
+    const double r = __fma_rn(-g, g, R.m);
+    // r as FP32 (its leading bits, 2^-86 <= |r| <= 2^-40 or 0), the correction in 2^-12 ulp
     const int rh = __double2hiint(r), rl = __double2loint(r);
     const int rb = ((__funnelshift_l(rl, rh, 3) & 0x7fffffff) | (rh & 0x80000000)) - 0x40000000;
     const float rf = (rh & 0x7fffffff) == 0 ? 0.f : __int_as_float(rb);
-    // + 1023: rounds to the nearest ulp by a shift
-    const int f = __float_as_int(__fmaf_rn(__fmul_rn(rf, yh), 9223372036854775808.f, 12582912.f)) - (0x4b400000 - 1023);
-    long long out = gb + (f >> 11);
-    if (((f + 3) & 2047) <= 4 || (unsigned)(e + 900) > 1800u) {
-        if ((unsigned)(e + 900) > 1800u) return __dsqrt_rn(x);
-        const double G = __longlong_as_double(out);
-        const long long Rb = bits64(__fma_rn(-G, G, m));
-        const long long ub = out - (52ll << 52);  // G * ulp(G), G in [1, 2)
-        const bool neg = Rb < 0;
-        const long long Rm = Rb & 0x7fffffffffffffffll;
-        // (G = 2, just above the largest root, stands at its lower neighbour's ulp)
-        const bool off = (neg ? Rm >= ub : Rm > ub) || (neg && (out & 0xfffffffffffffll) == 0 && Rm > 0);
-        if (off) out += neg ? -1 : 1;
+    // + 2047: rounds to the nearest ulp by a shift
+    const int f = __float_as_int(__fmaf_rn(__fmul_rn(rf, yh), 18446744073709551616.f, 12582912.f)) - (0x4b400000 - 2047);
+    R.out = gb + (f >> 12);
+    R.unsure = ((f + 3) & 4095) <= 4 || (unsigned)(e + 900) > 1800u;
+    return R;
+}
+__device__ __forceinline__ void root_decide(Root64 &R) {
+    if ((unsigned)((__double2hiint(R.x) >> 20) - 1023 + 900) > 1800u) {
+        R.out = __double_as_longlong(__dsqrt_rn(R.x));
+        R.qe = 0;
+        return;
     }
-    return __longlong_as_double(out + ((long long)qe << 32));
+    const double G = __longlong_as_double(R.out);
+    const long long Rb = bits64(__fma_rn(-G, G, R.m));
+    const long long ub = R.out - (52ll << 52);  // G * ulp(G), G in [1, 2)
+    const bool neg = Rb < 0;
+    const long long Rm = Rb & 0x7fffffffffffffffll;
+    // (G = 2, just above the largest root, stands at its lower neighbour's ulp)
+    const bool off = (neg ? Rm >= ub : Rm > ub) || (neg && (R.out & 0xfffffffffffffll) == 0 && Rm > 0);
+    if (off) R.out += neg ? -1 : 1;
+}
+__device__ __forceinline__ double sqrt_rn64(double x) {
+    Root64 R = root_start(x);
+    if (R.unsure) root_decide(R);
+    return R.value();
 }
 
 template <> struct Num<float> {
@@ -161,24 +182,42 @@ __device__ __forceinline__ float solve2(float a, float b, float rh, bool &two) {
     return two ? u2 : u1;
 }
 // FP64: eight operations on the FP64 pipe, the comparisons, the doubling and the
-// halving on the integer pipe.  r h = +inf (fixed nodes) takes the one-term
-// branch, which gives +inf too.
-__device__ __forceinline__ double solve2(double a, double b, double rh, bool &two) {
+// halving on the integer pipe; in two parts like the root.  r h = +inf (fixed
+// nodes) takes the one-term branch, which gives +inf too.
+struct Solve64 {
+    double ab, u1;
+    Root64 root;
+    bool two;
+};
+__device__ __forceinline__ Solve64 solve2_start(double a, double b, double rh) {
     using N = Num<double>;
+    Solve64 S;
     const double d = N::sub(a, b);
-    two = N::below(d, rh) && __double2hiint(rh) < 0x7ff00000;
+    S.two = N::below(d, rh) && __double2hiint(rh) < 0x7ff00000;
     // 2 r h by its exponent (exact; where r h is subnormal its square is 0 in any
     // case).  Not 2 (r h)^2: that loses the bits of a square just below the normal range.
     const double rh2 = __hiloint2double(__double2hiint(rh) + (1 << 20), __double2loint(rh));
     const double disc = N::sub(N::mul(rh2, rh), N::mul(d, d));
-    const double w = N::add(N::add(a, b), sqrt_rn64(two ? disc : 1.0));
+    S.root = root_start(S.two ? disc : 1.0);
+    S.ab = N::add(a, b);
+    S.u1 = N::add(N::mn(a, b), rh);
+    return S;
+}
+__device__ __forceinline__ double solve2_end(const Solve64 &S) {
+    using N = Num<double>;
+    const double w = N::add(S.ab, S.root.value());
     // w / 2 by its exponent, where that is exact (it always is but next to the
     // ends of the FP64 range)
     const int wh = __double2hiint(w);
     double u2 = __hiloint2double(wh - (1 << 20), __double2loint(w));
-    if (two && ((unsigned)(wh & 0x7fffffff) - (2u << 20)) >= ((0x7ffu - 2u) << 20)) u2 = N::mul(w, 0.5);
-    const double u1 = N::add(N::mn(a, b), rh);
-    return two ? u2 : u1;
+    if (S.two && ((unsigned)(wh & 0x7fffffff) - (2u << 20)) >= ((0x7ffu - 2u) << 20)) u2 = N::mul(w, 0.5);
+    return S.two ? u2 : S.u1;
+}
+__device__ __forceinline__ double solve2(double a, double b, double rh, bool &two) {
+    Solve64 S = solve2_start(a, b, rh);
+    if (S.root.unsure) root_decide(S.root);
+    two = S.two;
+    return solve2_end(S);
 }
 
 // 2-D Godunov local solve.  vm*/vp* are the neighbours on the minus/plus side
