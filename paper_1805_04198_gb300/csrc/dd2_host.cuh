@@ -15,6 +15,7 @@ struct DDPlan {
     size_t fine_smem, step1_smem, step4_smem;
     size_t fine_limit, step1_limit, step4_limit;  // what decides whether the size is supported
     int grid_threads;
+    int box_k;  // subdomains swept by one warp each (box2.cuh) with this many columns per lane; 0: by the engine
     bool adaptive;  // per-node weight: history of C_H and a fourth Alg. 5 static
 };
 
@@ -144,7 +145,9 @@ inline DDPlan dd_plan(const eik_grid *grid, const eik_dd_params *p) {
     auto sizes = [&](auto zero) {
         using T = decltype(zero);
         const int my = P.G.ncy + 1;
-        P.fine_smem = engine_smem_bytes<T, 1, false>(P.G.tnb, P.G.tny);
+        P.box_k = box2_use<T>(P.G.tnx, P.G.tny);
+        P.fine_smem = P.box_k ? box2_smem_bytes<T>(P.G.tnx, P.G.tny)
+                              : engine_smem_bytes<T, 1, false>(P.G.tnb, P.G.tny);
         P.step1_smem = engine_smem_bytes<T, 1, false>(gnb, my);
         P.step4_smem = P.adaptive ? engine_smem_bytes<T, 4, true>(gnb, my) : engine_smem_bytes<T, 3, true>(gnb, my);
         P.fine_limit = engine_limit_bytes<T, 1, false>(P.G.tnb, P.G.tny);

@@ -71,15 +71,10 @@ __global__ void k_fine_plan(DDArgs<T> A, int t0, int ntl) {
     }
 }
 
-// Subdomain kernel: with a plan, CTA b solves subdomain A.order[b] when b is
-// below the count of subdomains that need a solve; without one, CTA b
-// solves subdomain A.tile0 + b if its data changed.
+// Subdomain kernel: CTA b solves subdomain A.order[b] when b is below the count
+// of subdomains that need a solve.
 template <class T>
 __device__ __forceinline__ void k_fine_entry(const DDArgs<T> &A, char *smem) {
-    if (!A.order) {
-        k_fine_body<T>(A, smem, A.tile0 + blockIdx.x);
-        return;
-    }
     if (*A.done || (int)blockIdx.x >= *(volatile const int *)A.order_cnt) return;
     k_fine_body<T>(A, smem, A.order[blockIdx.x], false);
 }
@@ -90,6 +85,20 @@ __global__ void __maxnreg__(96) k_fine_f32(DDArgs<float> A) {
 __global__ void __maxnreg__(168) k_fine_f64(DDArgs<double> A) {
     extern __shared__ __align__(16) char smem[];
     k_fine_entry<double>(A, smem);
+}
+
+template <int K, class T>
+__global__ void __launch_bounds__(BOX2_THREADS) k_fine_box(DDArgs<T> A) {
+    extern __shared__ __align__(16) char smem[];
+    if (*A.done || (int)blockIdx.x >= *(volatile const int *)A.order_cnt) return;
+    k_fine_box_body<K, T>(A, smem, A.order[blockIdx.x], false);
+}
+
+template <class T>
+constexpr void (*fine_box_kernel(int k))(DDArgs<T>) {
+    if constexpr (box2_kmax<T>() > 2)
+        if (k > 2) return k == 3 ? k_fine_box<3, T> : k_fine_box<4, T>;
+    return k == 1 ? k_fine_box<1, T> : k_fine_box<2, T>;
 }
 
 template <class T> struct DDKernels;
@@ -202,6 +211,7 @@ struct DDSolve {
     int nsm = 0, ew = 256, eb = 0, tb = 0, ntiles = 0, fine_threads = 0;
     size_t fine_smem = 0;
     void (*step4k)(DDArgs<T>) = nullptr;
+    void (*finek)(DDArgs<T>) = nullptr;
     long long nl = 0;  // launches made
 
     int setup(const eik_grid *grid, const void *r, const uint8_t *gamma, const void *g, const eik_dd_params *p,
@@ -243,7 +253,12 @@ struct DDSolve {
                       P.step4_limit, smem_optin);
             return EIK_EUNSUPPORTED;
         }
-        if ((rc = cuda_check(set_dyn_smem(DDKernels<T>::fine, (int)fine_smem), "smem attr fine")))
+        finek = DDKernels<T>::fine;
+        if (P.box_k) {
+            finek = fine_box_kernel<T>(P.box_k);
+            fine_threads = BOX2_THREADS;
+        }
+        if ((rc = cuda_check(set_dyn_smem(finek, (int)fine_smem), "smem attr fine")))
             return rc;
         if ((rc = cuda_check(set_dyn_smem(DDKernels<T>::step1, (int)P.step1_smem), "smem attr step1")))
             return rc;
@@ -273,7 +288,10 @@ struct DDSolve {
     int start() {
         const DDGeom &G = P.G;
         EIK_LAUNCH("dd_init", s, k_init_stats<T><<<1, 256, 0, s>>>(A)); ++nl;
-        EIK_LAUNCH("dd_pack_tiles", s, k_pack_tiles<T><<<tb, ew, 0, s>>>(A)); ++nl;
+        if (!P.box_k) {
+            EIK_LAUNCH("dd_pack_tiles", s, k_pack_tiles<T><<<tb, ew, 0, s>>>(A));
+            ++nl;
+        }
         EIK_LAUNCH("dd_pack_coarse", s, k_pack_coarse<T><<<eb, ew, 0, s>>>(A)); ++nl;
         EIK_LAUNCH("dd_step1_coarse_fsm", s, DDKernels<T>::step1<<<G.ngrids, P.grid_threads, P.step1_smem, s>>>(A));
         ++nl;
@@ -284,7 +302,7 @@ struct DDSolve {
     int fine(int t0, int t1) {
         if (t1 <= t0) return EIK_OK;
         EIK_LAUNCH("dd_fine_plan", s, k_fine_plan<T><<<t1 - t0, 256, 0, s>>>(A, t0, t1 - t0)); ++nl;
-        EIK_LAUNCH("dd_fine_subdomains", s, DDKernels<T>::fine<<<t1 - t0, fine_threads, fine_smem, s>>>(A)); ++nl;
+        EIK_LAUNCH("dd_fine_subdomains", s, finek<<<t1 - t0, fine_threads, fine_smem, s>>>(A)); ++nl;
         return EIK_OK;
     }
 

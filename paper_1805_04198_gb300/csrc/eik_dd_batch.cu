@@ -259,6 +259,21 @@ __device__ __forceinline__ void kb_fine_body(const DDArgs<T> &A, char *smem, int
     k_fine_body<T>(A, smem, tile);
 }
 EIK_BATCH_PAIR(kb_fine, kb_fine_body, 112, 168)
+template <int K, class T>
+__global__ void __launch_bounds__(BOX2_THREADS) kb_fine_box(const DDArgs<T> *__restrict__ args, ItemList L) {
+    extern __shared__ __align__(16) char smem[];
+    for_items(L, [&](int p, int local) {
+        const DDArgs<T> A = args[p];
+        k_fine_box_body<K, T>(A, smem, local);
+    });
+}
+
+template <class T>
+constexpr void (*fine_box_kernel(int k))(const DDArgs<T> *, ItemList) {
+    if constexpr (box2_kmax<T>() > 2)
+        if (k > 2) return k == 3 ? kb_fine_box<3, T> : kb_fine_box<4, T>;
+    return k == 1 ? kb_fine_box<1, T> : kb_fine_box<2, T>;
+}
 
 template <class T> struct BatchKernels;
 template <> struct BatchKernels<float> {
@@ -281,6 +296,7 @@ constexpr int ELEM_BLOCK = 256;  // threads (and elements) per element-stage blo
 
 struct BoxClass {
     int nw;           // warps per CTA (32-column blocks of the widest box)
+    int box_k;        // subdomains: columns per lane of the one-warp form, 0: by the engine
     size_t smem;      // dynamic shared memory (max over the class)
     int n, items;     // problems, boxes
     int prob_at, pre_at;  // offsets of the tables in the int area
@@ -369,7 +385,7 @@ static void batch_plan(int nprob, const eik_grid *grids, const eik_dd_params *pa
     auto blocks = [](size_t n) { return (n + ELEM_BLOCK - 1) / ELEM_BLOCK; };
     B.tiles_at = push_prefix([&](int p) {
         const DDGeom &G = B.P[p].G;
-        return blocks((size_t)G.tx * G.ty * G.tnx * G.tny);
+        return B.P[p].box_k ? 0 : blocks((size_t)G.tx * G.ty * G.tnx * G.tny);
     });
     B.tiles_total = B.tab.back();
     B.coarse_at = push_prefix([&](int p) { return blocks(B.P[p].G.coarse_elems); });
@@ -392,7 +408,8 @@ static void batch_plan(int nprob, const eik_grid *grids, const eik_dd_params *pa
         for (int p = 0; p < nprob; ++p) cst[p] = cost(p);
         for (int w : uk) {
             BoxClass c;
-            c.nw = w;
+            c.box_k = w >= 1000 ? w - 1000 : 0;
+            c.nw = c.box_k ? BOX2_THREADS / 32 : w;
             c.smem = 0;
             std::vector<int> ids;
             for (int p = 0; p < nprob; ++p)
@@ -417,7 +434,7 @@ static void batch_plan(int nprob, const eik_grid *grids, const eik_dd_params *pa
         }
     };
     make_classes(
-        B.fine, [&](int p) { return B.P[p].G.tnb; },
+        B.fine, [&](int p) { return B.P[p].box_k ? 1000 + B.P[p].box_k : B.P[p].G.tnb; },
         [&](int p) { return B.P[p].G.tx * B.P[p].G.ty; },
         [&](int p) { return (long long)B.P[p].G.tnx * B.P[p].G.tny; }, [&](int p) { return B.P[p].fine_smem; });
     make_classes(
@@ -500,8 +517,7 @@ static int batch_run(int nprob, const eik_grid *grids, const void *const *r, con
     int nsm = 0, smem_optin = 0;
     if ((rc = cuda_check(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev), "attr"))) return rc;
     cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    size_t need_fine = 0, need_grid = 0;
-    for (auto &c : B.fine) need_fine = std::max(need_fine, c.smem);
+    size_t need_grid = 0;
     for (auto &c : B.grid) need_grid = std::max(need_grid, c.smem);
     size_t limit_fine = 0, limit_grid = 0;
     for (auto &P : B.P) {
@@ -512,8 +528,13 @@ static int batch_run(int nprob, const eik_grid *grids, const void *const *r, con
         set_error("shared memory need (%zu, %zu) exceeds the device limit %d", limit_fine, limit_grid, smem_optin);
         return EIK_EUNSUPPORTED;
     }
-    if ((rc = cuda_check(set_dyn_smem(BatchKernels<T>::fine, (int)std::max<size_t>(need_fine, 1)), "smem attr fine")))
-        return rc;
+    auto finek = [](const BoxClass &c) { return c.box_k ? fine_box_kernel<T>(c.box_k) : BatchKernels<T>::fine; };
+    for (auto it = B.fine.begin(); it != B.fine.end(); ++it) {
+        size_t need = it->smem;
+        for (auto &c : B.fine)
+            if (finek(c) == finek(*it)) need = std::max(need, c.smem);
+        if ((rc = cuda_check(set_dyn_smem(finek(*it), (int)need), "smem attr fine"))) return rc;
+    }
     if ((rc = cuda_check(set_dyn_smem(BatchKernels<T>::step1, (int)std::max<size_t>(need_grid, 1)), "smem attr step1")))
         return rc;
     if ((rc = cuda_check(set_dyn_smem(step4k, (int)std::max<size_t>(need_grid, 1)), "smem attr step4")))
@@ -578,7 +599,7 @@ static int batch_run(int nprob, const eik_grid *grids, const void *const *r, con
     for (int k = 0; k <= B.max_iter; ++k) {
         for (const BoxClass &c : B.fine) {
             EIK_LAUNCH("dd_fine_subdomains", s,
-                       BatchKernels<T>::fine<<<ctas(BatchKernels<T>::fine, c, fq), 32 * c.nw, c.smem, s>>>(dargs, item_list(c, fq)));
+                       finek(c)<<<ctas(finek(c), c, fq), 32 * c.nw, c.smem, s>>>(dargs, item_list(c, fq)));
             ++nl;
         }
         EIK_LAUNCH("dd_alg4_restrict", s, kb_alg4<T><<<eb, ELEM_BLOCK, 0, s>>>(dargs, coarse, k)); ++nl;

@@ -321,6 +321,35 @@ struct FsmPolicy {
         changed = Num<T>::lt(ut, self);
         return changed ? ut : self;
     }
+    // K independent nodes; their FP64 roots run together
+    template <int K>
+    __device__ __forceinline__ void update_all(const float *self, const float *a, const float *b, const float *rh,
+                                               bool *changed, float *v) const {
+#pragma unroll
+        for (int j = 0; j < K; ++j) v[j] = update(self[j], a[j], b[j], rh[j], changed[j]);
+    }
+    template <int K>
+    __device__ __forceinline__ void update_all(const double *self, const double *a, const double *b,
+                                               const double *rh, bool *changed, double *v) const {
+        Solve64 S[K];
+        bool unsure = false;
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            S[j] = solve2_start(a[j], b[j], rh[j]);
+            unsure = unsure || S[j].root.unsure;
+        }
+        if (unsure) {
+#pragma unroll
+            for (int j = 0; j < K; ++j)
+                if (S[j].root.unsure) root_decide(S[j].root);
+        }
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            const double ut = solve2_end(S[j]);
+            changed[j] = Num<double>::lt(ut, self[j]);
+            v[j] = changed[j] ? ut : self[j];
+        }
+    }
 };
 
 // Shared memory of one warp (32-bit shared addresses).

@@ -46,3 +46,32 @@ def test_ranges(gpu, scale, g0):
     u_ref, _, _ = O.fsm(r, gamma, g, 0.05)
     u, _ = _fsm(gpu, r, gamma, g, 0.05)
     np.testing.assert_array_equal(u, u_ref)
+
+
+# Small subdomains, which one warp sweeps with K columns a lane: widths around the 32 K edges, heights from the
+# smallest to the largest that the form takes, and the first ones that go to the engine (FP32: 128 columns by 99
+# rows; FP64: 64 columns).
+@pytest.mark.parametrize("tiles,cells,c", [((1, 1), (2, 2), 1), ((3, 2), (2, 6), 2), ((2, 2), (30, 4), 2), ((2, 1), (31, 31), 31),
+                                           ((1, 2), (32, 40), 4), ((2, 2), (62, 2), 2), ((1, 2), (63, 63), 21),
+                                           ((2, 2), (64, 8), 8)])
+def test_small_boxes(gpu, tiles, cells, c):
+    shape = tuple(t * s + 1 for t, s in zip(reversed(tiles), reversed(cells)))
+    r, gamma, g = _problem(shape, 5 + sum(shape), g0=-1.0 if cells[1] == 4 else 0.0)
+    kw = dict(theta=0.2, max_iter=3, tol=0.0, max_coarse_sweeps=8)
+    u_ref, s_ref, _ = O.dd(r, gamma, g, 0.05, tiles, c, **kw)
+    u, st = gpu.dd_solve(*(torch.from_numpy(a).to(DEV) for a in (r, gamma, g)), 0.05, tiles, c, **kw)
+    assert st["iters"] == s_ref["iters"]
+    np.testing.assert_array_equal(u.cpu().numpy(), u_ref)
+
+
+# FP32: a single subdomain has no inflow, so off the coarse lines it holds what plain sweeping gives
+@pytest.mark.parametrize("nx,ny,c", [(3, 3, 2), (17, 9, 8), (32, 32, 31), (33, 5, 2), (64, 22, 21), (65, 129, 16), (96, 20, 19),
+                                     (97, 33, 32), (127, 97, 6), (127, 100, 9), (129, 65, 32)])
+def test_small_boxes_f32(gpu, nx, ny, c):
+    r, gamma, g = _problem((ny, nx), nx + 3 * ny)
+    u_ref, st_ref = _fsm(gpu, r, gamma, g, 0.05, torch.float32)
+    u, st = gpu.dd_solve(torch.from_numpy(r).to(DEV, torch.float32), torch.from_numpy(gamma).to(DEV),
+                         torch.from_numpy(g).to(DEV, torch.float32), 0.05, (1, 1), c, max_iter=2)
+    off = (np.arange(ny)[:, None] % c != 0) & (np.arange(nx)[None, :] % c != 0)
+    np.testing.assert_array_equal(u.cpu().numpy()[off], u_ref[off])
+    assert st["fsm_sweeps_max"] == st_ref["sweeps"]
