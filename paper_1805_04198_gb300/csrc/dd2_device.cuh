@@ -729,7 +729,7 @@ __device__ __forceinline__ void k_fine_body(const DDArgs<T> &A, char *smem, int 
 // first warp (box2.cuh, K columns per lane).  r, Gamma and g come from the
 // caller's arrays, so nothing of it is packed.  Bound by the chain of one step
 // (a dependent local solve and two shuffles); the subdomain stage of a 501^2
-// FP32 solve with 10 x 10 boxes of 51^2, 31 passes: 2.4 ms, by the engine 5.1 ms.
+// FP32 solve with 10 x 10 boxes of 51^2, 31 passes: 2.4 ms, by the engine 6.0 ms.
 template <int K, class T>
 __device__ __forceinline__ void k_fine_box_body(const DDArgs<T> &A, char *smem, int tile, bool check = true) {
     if (*A.done) return;

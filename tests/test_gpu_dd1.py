@@ -148,3 +148,20 @@ def test_expired_barrier_reports_timeout_then_solves_exactly():
     u, st = _gpu(r, gam, g, h, N, M, torch.float64, **kw)
     assert st["error"] == 0
     np.testing.assert_array_equal(u.cpu().numpy(), u_o)
+
+
+# the subintervals' positions are checked 32 at a time by 8 lanes, the coarse nodes 32 at a time by a warp, and
+# subintervals that do not fit shared memory stay in global memory: one below, at and above each of these
+@pytest.mark.parametrize("N,M", [(1, 1), (2, 6), (31, 7), (32, 8), (33, 31), (5, 32), (3, 62), (64, 63), (153, 64), (700, 33),
+                                 (1217, 10), (2, 13000), (2, 15000), (149, 7000)])
+def test_block_edges_bitwise(N, M):
+    r, gam, g, h = _random(N, M, 100 + N + M, [0, N * M, (N * M) // 3])
+    if N > 3:  # a node that no wave enters, and negative boundary values
+        r[M + M // 2] = np.inf
+        g[0] = -0.7
+    kw = dict(theta=0.8 if M % 2 else 1.0, max_iter=6, max_coarse_sweeps=1000)
+    u_o, st_o, _ = O.dd1(r, gam, g, h, N, M, **kw)
+    u, st = _gpu(r, gam, g, h, N, M, torch.float64, **kw)
+    np.testing.assert_array_equal(u.cpu().numpy(), u_o)
+    for k in STAT_KEYS:
+        assert st[k] == st_o[k], (k, st[k], st_o[k])
