@@ -366,7 +366,9 @@ int eik_dd_batched_autotune(int nprob, const eik_grid *grids, const void *const 
  * GPU that loads the library keeps until the process exits.  This entry point
  * has no counterpart in the paper; it only changes where the scratch lives.
  *  - Problems whose eik_dd_workspace_size exceeds the array are rejected with
- *    EIK_ENOMEM before any work is enqueued.
+ *    EIK_ENOMEM before any work is enqueued; 3-D problems only if they do not
+ *    fit without the optional part of it (packed subdomains and line flags)
+ *    either.
  *  - The first call on a device looks up the array's device address (a
  *    cudaGetSymbolAddress call, made once per device with that device
  *    current); make that first call before any stream capture.

@@ -119,10 +119,10 @@ template <> struct DDKernels<double> {
 // Host side
 // --------------------------------------------------------------------------
 // 3-D implementation (eik_dd3.cu)
-size_t dd3_workspace_size(const eik_grid *grid, const eik_dd_params *p);
+size_t dd3_workspace_size(const eik_grid *grid, const eik_dd_params *p, bool lean);
 bool dd3_validate(const eik_grid *grid, const eik_dd_params *p);
 int dd3_run(const eik_grid *grid, const void *r, const uint8_t *gamma, const void *g, const eik_dd_params *p,
-            void *u_out, void *ws, eik_dd_stats *stats, cudaStream_t s);
+            void *u_out, void *ws, size_t ws_bytes, eik_dd_stats *stats, cudaStream_t s);
 // 1-D implementation (eik_dd1.cu)
 bool dd1_validate(const eik_grid *grid, const eik_dd_params *p);
 size_t dd1_workspace_size(const eik_grid *grid, const eik_dd_params *p);
@@ -361,8 +361,13 @@ using namespace eik;
 extern "C" size_t eik_dd_workspace_size(const eik_grid *grid, const eik_dd_params *params) {
     if (!dd_validate(grid, params)) return 0;
     if (grid->ndim == 1) return dd1_workspace_size(grid, params);
-    if (grid->ndim == 3) return dd3_workspace_size(grid, params);
+    if (grid->ndim == 3) return dd3_workspace_size(grid, params, false);
     return dd_plan(grid, params).bytes;
+}
+
+// The least workspace that a valid request runs with.
+static size_t dd_least_workspace(const eik_grid *grid, const eik_dd_params *params) {
+    return grid->ndim == 3 ? dd3_workspace_size(grid, params, true) : eik_dd_workspace_size(grid, params);
 }
 
 extern "C" int eik_dd_solve(const eik_grid *grid, const void *r, const uint8_t *gamma, const void *g,
@@ -377,16 +382,14 @@ extern "C" int eik_dd_solve(const eik_grid *grid, const void *r, const uint8_t *
         set_error("workspace must be 256-byte aligned");
         return EIK_EINVAL;
     }
-    const size_t need = grid->ndim == 1   ? dd1_workspace_size(grid, params)
-                        : grid->ndim == 3 ? dd3_workspace_size(grid, params)
-                                          : dd_plan(grid, params).bytes;
+    const size_t need = dd_least_workspace(grid, params);
     if (ws_bytes < need) {
         set_error("workspace of %zu bytes is smaller than the %zu required", ws_bytes, need);
         return EIK_ENOMEM;
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (grid->ndim == 1) return dd1_run(grid, r, gamma, g, params, u_out, ws, stats, s);
-    if (grid->ndim == 3) return dd3_run(grid, r, gamma, g, params, u_out, ws, stats, s);
+    if (grid->ndim == 3) return dd3_run(grid, r, gamma, g, params, u_out, ws, ws_bytes, stats, s);
     if (grid->dtype == EIK_F64) return dd_run<double>(grid, r, gamma, g, params, u_out, ws, stats, s);
     return dd_run<float>(grid, r, gamma, g, params, u_out, ws, stats, s);
 }
@@ -609,8 +612,8 @@ static int scratch_address(void **out) {
 
 extern "C" int eik_dd_solve_noalloc(const eik_grid *grid, const void *r, const uint8_t *gamma, const void *g,
                                     const eik_dd_params *params, void *u_out, eik_dd_stats *stats, void *stream) {
-    const size_t need = eik_dd_workspace_size(grid, params);
-    if (need == 0) return EIK_EINVAL;
+    if (!dd_validate(grid, params)) return EIK_EINVAL;
+    const size_t need = dd_least_workspace(grid, params);
     if (need > (size_t)EIK_NOALLOC_SCRATCH_BYTES) {
         set_error("eik_dd_solve_noalloc: problem needs %zu bytes of scratch, the static scratch holds %zu; "
                   "use eik_dd_solve with a caller workspace",

@@ -50,7 +50,7 @@ struct DD3Args {
     const T *g;
     T *u_out;
     long long sy, sz;
-    T *rp;            // r h of the subdomains, [subdomain][column tile][z][32]
+    T *rp;            // r h of the subdomains, [subdomain][column tile][z][32]; null without room for it
     int fpx, fps, fo, gpx, gps, go;  // layout (see Box3) of the subdomain and the shifted-grid boxes
     Grid3 *grids;
     int *offmap;  // [c^3] offset -> grid index (-1 if not a shifted grid)
@@ -61,7 +61,7 @@ struct DD3Args {
     int *done;
     double *deltas;
     int *chg;
-    uint8_t *lflag;  // causal sweep: lines to walk again
+    uint8_t *lflag;  // causal sweep: lines to walk again; null without room: all of them
     unsigned *bar;
     DevStats3 *st;
     // Step 2 data of each subdomain's last solve in this call (the starting
@@ -404,6 +404,28 @@ struct Fsm3Tile : Fsm3Update<T> {
         ldg_if(on, rp + c.at + ahead * c.step, v);
     }
 };
+// The same from the caller's arrays, for a workspace without room for the packed
+// copy (73^3 FP64, 3^3 subdomains of 25^3: 89 ms a solve, packed 74 ms).
+template <class T>
+struct Fsm3Direct : Fsm3Update<T> {
+    const T *r;  // at the subdomain's first node
+    const uint8_t *gamma;
+    long long sy, sz;
+    T h;
+    struct Cursor {
+        long long at, step;
+    };
+    __device__ __forceinline__ Cursor cursor(int x, int y, int, int, int z0, int dz, int kp0) const {
+        return Cursor{x + y * sy + (z0 + (long long)kp0 * dz) * sz, dz * sz};
+    }
+    __device__ __forceinline__ void advance(Cursor &c) const { c.at += c.step; }
+    __device__ __forceinline__ void load_if(bool on, const Cursor &c, int ahead, T &v) const {
+        if (on) {
+            const long long f = c.at + ahead * c.step;
+            v = !gamma[f] && r[f] > T(0) ? Num<T>::mul(r[f], h) : Num<T>::inf();
+        }
+    }
+};
 // r of a shifted grid in box order (<= 0 at fixed nodes)
 template <class T>
 struct Fsm3Grid : Fsm3Update<T> {
@@ -695,7 +717,7 @@ __device__ __forceinline__ bool same_bits3<double>(double a, double b) {
     return __double_as_longlong(a) == __double_as_longlong(b);
 }
 
-template <class T>
+template <class T, bool PACKED>
 __global__ void __launch_bounds__(BOX3_THREADS, 1) k3_fine(DD3Args<T> A) {
     if (*A.done) return;
     extern __shared__ __align__(16) char smem[];
@@ -754,12 +776,23 @@ __global__ void __launch_bounds__(BOX3_THREADS, 1) k3_fine(DD3Args<T> A) {
     }
     if (threadIdx.x == 0) A.sig_ok[tile] = 1;
     __syncthreads();
-    Fsm3Tile<T> pol;
-    pol.rp = A.rp + (size_t)tile * box3_tiles(mx, my) * mz * 32;
-    pol.mz = mz;
     long long sweeps;
     bool conv;
-    box3_sweeps(B, pol, A.max_fsm, sweeps, conv);
+    if constexpr (PACKED) {
+        Fsm3Tile<T> pol;
+        pol.rp = A.rp + (size_t)tile * box3_tiles(mx, my) * mz * 32;
+        pol.mz = mz;
+        box3_sweeps(B, pol, A.max_fsm, sweeps, conv);
+    } else {
+        Fsm3Direct<T> pol;
+        const size_t f = fidx(A, b0, b1, b2);
+        pol.r = A.r + f;
+        pol.gamma = A.gamma + f;
+        pol.sy = A.sy;
+        pol.sz = A.sz;
+        pol.h = T(G.h);
+        box3_sweeps(B, pol, A.max_fsm, sweeps, conv);
+    }
     if (threadIdx.x == 0) {
         atomicMax(&A.st->fsm_sweeps_max, (unsigned long long)sweeps);
         if (!conv) atomicAdd(&A.st->fsm_caps, 1ull);
@@ -1017,7 +1050,7 @@ __device__ bool causal3_line(const DD3Args<T> &A, int e, const int *X, int rev) 
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {  // the line along a through the node, if it is one
                         const int b1 = a == 0 ? 1 : 0, b2 = a == 2 ? 1 : 2;
-                        if (a != e && (Y[b1] % c == 0 || Y[b2] % c == 0)) A.lflag[line3_flag(G, a, Y)] = 1;
+                        if (A.lflag && a != e && (Y[b1] % c == 0 || Y[b2] % c == 0)) A.lflag[line3_flag(G, a, Y)] = 1;
                     }
                 }
                 pred = u[q];
@@ -1035,7 +1068,8 @@ __global__ void k3_causal(DD3Args<T> A, int only_if_not_done) {
     const int lane = threadIdx.x & 31;
     __shared__ int blk_changed;
     if (blockIdx.x == 0 && threadIdx.x < 3) A.chg[threadIdx.x] = 0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < line3_flags(G); i += (size_t)gridDim.x * blockDim.x)
+    const size_t nflags = A.lflag ? line3_flags(G) : 0;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nflags; i += (size_t)gridDim.x * blockDim.x)
         A.lflag[i] = 0;
     if (!grid_barrier(A.bar, &A.st->err, wlim)) return;
     int rounds = 0;
@@ -1051,9 +1085,11 @@ __global__ void k3_causal(DD3Args<T> A, int only_if_not_done) {
                 lines.get(L, xf, xs);
 #pragma unroll
                 for (int a = 0; a < 3; ++a) X[a] = a == lines.fast ? xf : (a == lines.slow ? xs : 0);
-                uint8_t *flag = A.lflag + line3_flag(G, e, X);
-                if (rounds > 0 && !__ldcg(flag)) continue;
-                *flag = 0;
+                if (A.lflag) {
+                    uint8_t *flag = A.lflag + line3_flag(G, e, X);
+                    if (rounds > 0 && !__ldcg(flag)) continue;
+                    *flag = 0;
+                }
                 const bool fwd = causal3_line(A, e, X, 0);
                 const bool back = causal3_line(A, e, X, 1);
                 ch = ch || fwd || back;
@@ -1155,8 +1191,9 @@ static bool dd3_plan(const eik_grid *grid, const eik_dd_params *p, DD3Plan &P) {
     return true;
 }
 
+// lean: without the packed subdomains and the line flags, a fifth less
 template <class T>
-static size_t dd3_layout(const DD3Plan &P, DD3Args<T> *A, void *ws, int max_iter) {
+static size_t dd3_layout(const DD3Plan &P, DD3Args<T> *A, void *ws, int max_iter, bool lean) {
     const DD3Geom &G = P.G;
     Carver cv(ws);
     T *U = cv.take<T>(G.nc), *Uprev = cv.take<T>(G.nc), *U0 = cv.take<T>(G.nc), *rc = cv.take<T>(G.nc);
@@ -1169,14 +1206,14 @@ static size_t dd3_layout(const DD3Plan &P, DD3Args<T> *A, void *ws, int max_iter
     int *done = cv.take<int>(4);
     double *deltas = cv.take<double>((size_t)max_iter + 2);
     int *chg = cv.take<int>(4);
-    uint8_t *lflag = cv.take<uint8_t>(line3_flags(G));
+    uint8_t *lflag = lean ? nullptr : cv.take<uint8_t>(line3_flags(G));
     unsigned *bar = cv.take<unsigned>(4);
     DevStats3 *st = cv.take<DevStats3>(1);
     const size_t ntl = (size_t)G.T[0] * G.T[1] * G.T[2], nsl = (size_t)box3_face_slots(G.S);
     T *sig_u = cv.take<T>(ntl * nsl);
     uint8_t *sig_w = cv.take<uint8_t>(ntl * nsl);
     int *sig_ok = cv.take<int>(ntl);
-    T *rp = cv.take<T>(ntl * box3_tiles(G.S[0] + 1, G.S[1] + 1) * (G.S[2] + 1) * 32);
+    T *rp = lean ? nullptr : cv.take<T>(ntl * box3_tiles(G.S[0] + 1, G.S[1] + 1) * (G.S[2] + 1) * 32);
     T *Ch[4] = {nullptr, nullptr, nullptr, nullptr}, *th = nullptr;
     double *du = nullptr;
     if (P.adaptive) {
@@ -1232,11 +1269,12 @@ __global__ void k3_tables(Grid3 *grids, int *offmap, int c, int n0, int n1, int 
             }
 }
 
-size_t dd3_workspace_size(const eik_grid *grid, const eik_dd_params *p) {
+// lean = false: the workspace to ask for; true: what a solve can do with
+size_t dd3_workspace_size(const eik_grid *grid, const eik_dd_params *p, bool lean) {
     DD3Plan P;
     dd3_plan(grid, p, P);
-    return grid->dtype == EIK_F64 ? dd3_layout<double>(P, nullptr, nullptr, p->max_iter)
-                                  : dd3_layout<float>(P, nullptr, nullptr, p->max_iter);
+    return grid->dtype == EIK_F64 ? dd3_layout<double>(P, nullptr, nullptr, p->max_iter, lean)
+                                  : dd3_layout<float>(P, nullptr, nullptr, p->max_iter, lean);
 }
 
 bool dd3_validate(const eik_grid *grid, const eik_dd_params *p) {
@@ -1259,7 +1297,8 @@ bool dd3_validate(const eik_grid *grid, const eik_dd_params *p) {
 
 template <class T>
 static int dd3_run_t(const eik_grid *grid, const void *r, const uint8_t *gamma, const void *g,
-                     const eik_dd_params *p, void *u_out, void *ws, eik_dd_stats *stats, cudaStream_t s) {
+                     const eik_dd_params *p, void *u_out, void *ws, size_t ws_bytes, eik_dd_stats *stats,
+                     cudaStream_t s) {
     DD3Plan P;
     dd3_plan(grid, p, P);
     DD3Args<T> A;
@@ -1271,7 +1310,8 @@ static int dd3_run_t(const eik_grid *grid, const void *r, const uint8_t *gamma, 
     A.u_out = static_cast<T *>(u_out);
     A.sy = grid->stride[1];
     A.sz = grid->stride[2];
-    dd3_layout<T>(P, &A, ws, p->max_iter);
+    const bool lean = ws_bytes < dd3_layout<T>(P, nullptr, nullptr, p->max_iter, false);
+    dd3_layout<T>(P, &A, ws, p->max_iter, lean);
     A.theta = (T)p->theta;
     A.tol = (T)p->tol;
     A.max_iter = p->max_iter;
@@ -1294,7 +1334,8 @@ static int dd3_run_t(const eik_grid *grid, const void *r, const uint8_t *gamma, 
                   P.grid_limit, optin);
         return EIK_EUNSUPPORTED;
     }
-    if ((rc = cuda_check(set_dyn_smem(k3_fine<T>, (int)P.fine_smem), "attr")))
+    void (*const fine)(DD3Args<T>) = lean ? k3_fine<T, false> : k3_fine<T, true>;
+    if ((rc = cuda_check(set_dyn_smem(fine, (int)P.fine_smem), "attr")))
         return rc;
     if ((rc = cuda_check(set_dyn_smem(k3_step1<T>, (int)P.grid_smem), "attr")))
         return rc;
@@ -1313,7 +1354,10 @@ static int dd3_run_t(const eik_grid *grid, const void *r, const uint8_t *gamma, 
     EIK_LAUNCH("dd3_init", s, k3_init<T><<<1, 256, 0, s>>>(A)); ++nl;
     EIK_LAUNCH("dd3_tables", s, k3_tables<<<1, 32, 0, s>>>(A.grids, A.offmap, G.c, G.n[0], G.n[1], G.n[2])); ++nl;
     EIK_LAUNCH("dd3_pack_coarse", s, k3_pack_coarse<T><<<cgrid, ew, 0, s>>>(A)); ++nl;
-    EIK_LAUNCH("dd3_pack_tiles", s, k3_pack_tiles<T><<<ntiles, ew, 0, s>>>(A)); ++nl;
+    if (!lean) {
+        EIK_LAUNCH("dd3_pack_tiles", s, k3_pack_tiles<T><<<ntiles, ew, 0, s>>>(A));
+        ++nl;
+    }
     EIK_LAUNCH("dd3_step1_coarse_fsm", s, k3_step1<T><<<G.ng, P.grid_threads, P.grid_smem, s>>>(A)); ++nl;
     auto launch_causal = [&](int only) -> int {
         void *args[] = {&A, &only};
@@ -1326,7 +1370,7 @@ static int dd3_run_t(const eik_grid *grid, const void *r, const uint8_t *gamma, 
     };
     if ((rc = launch_causal(0))) return rc;
     for (int k = 0; k <= p->max_iter; ++k) {
-        EIK_LAUNCH("dd3_fine_subdomains", s, k3_fine<T><<<ntiles, P.fine_threads, P.fine_smem, s>>>(A)); ++nl;
+        EIK_LAUNCH("dd3_fine_subdomains", s, fine<<<ntiles, P.fine_threads, P.fine_smem, s>>>(A)); ++nl;
         EIK_LAUNCH("dd3_alg4_restrict", s, k3_alg4<T><<<cgrid, ew, 0, s>>>(A)); ++nl;
         EIK_LAUNCH("dd3_check", s, k3_check<T><<<1, 1, 0, s>>>(A, k)); ++nl;
         if (k == p->max_iter) break;
@@ -1343,9 +1387,9 @@ static int dd3_run_t(const eik_grid *grid, const void *r, const uint8_t *gamma, 
 }
 
 int dd3_run(const eik_grid *grid, const void *r, const uint8_t *gamma, const void *g, const eik_dd_params *p,
-            void *u_out, void *ws, eik_dd_stats *stats, cudaStream_t s) {
-    if (grid->dtype == EIK_F64) return dd3_run_t<double>(grid, r, gamma, g, p, u_out, ws, stats, s);
-    return dd3_run_t<float>(grid, r, gamma, g, p, u_out, ws, stats, s);
+            void *u_out, void *ws, size_t ws_bytes, eik_dd_stats *stats, cudaStream_t s) {
+    if (grid->dtype == EIK_F64) return dd3_run_t<double>(grid, r, gamma, g, p, u_out, ws, ws_bytes, stats, s);
+    return dd3_run_t<float>(grid, r, gamma, g, p, u_out, ws, ws_bytes, stats, s);
 }
 
 }  // namespace eik

@@ -45,3 +45,22 @@ def test_dd3_boxes(gpu, tiles, cells, c):
     u, st = gpu.dd_solve(*_dev(r, gamma, g), 0.05, tiles, c, **kw)
     assert st["iters"] == s_ref["iters"]
     np.testing.assert_array_equal(u.cpu().numpy(), u_ref)
+
+
+def test_dd3_without_room_for_packed_boxes(gpu):
+    """A problem that fits the library's static scratch only without the packed subdomains and the line flags: the
+    same solve, bit for bit."""
+    r, gamma, g = _problem((73, 73, 73), 3)
+    r[20:40, 10:30, 33] = np.inf
+    kw = dict(theta=0.2, max_iter=2, tol=0.0, max_coarse_sweeps=8)
+    R, G, g_t = _dev(r, gamma, g)
+    grid, p = gpu.make_grid(R, 0.05), gpu.dd_params((3, 3, 3), 4, **kw)
+    assert gpu.eik_dd_workspace_size(grid, p) > 32 << 20
+    u_ref, s_ref = gpu.dd_solve(R, G, g_t, 0.05, (3, 3, 3), 4, **kw)
+    u = torch.empty_like(R)
+    st = torch.zeros(gpu.ctypes.sizeof(gpu.DDStats), dtype=torch.uint8, device=DEV)
+    gpu.eik_dd_solve_noalloc(grid, R, G, g_t, p, u, st)
+    torch.cuda.synchronize()
+    got = gpu.parse_dd_stats(st)
+    assert torch.equal(u, u_ref)
+    assert {k: v for k, v in got.items() if k != "launches"} == {k: v for k, v in s_ref.items() if k != "launches"}
