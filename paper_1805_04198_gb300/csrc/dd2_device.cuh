@@ -1018,10 +1018,10 @@ __device__ void delta_body(const DDArgs<T> &A, int k, size_t bid, size_t nbid) {
     const DDGeom &G = A.G;
     double m = 0.0;
     for (size_t a = bid * blockDim.x + threadIdx.x; a < G.coarse_elems; a += nbid * blockDim.x) {
-        int g, i, j;
-        if (!coarse_decode(G, a, g, i, j)) continue;
         const T u1 = A.U[a], u0 = A.Uprev[a];
         if (u1 == u0) continue;
+        int g, i, j;
+        if (!coarse_decode(G, a, g, i, j)) continue;  // padding
         const double dv = fabs((double)u1 - (double)u0);
         if (dv > m) m = dv;
     }
