@@ -128,29 +128,15 @@ __global__ void k_adj_nodes(AdjArgs<T> A) {
     adj_nodes_body(A, blockIdx.x, gridDim.x);
 }
 
-// Skewed statics in storage order, 16 bytes of every channel per thread
-// ([dir][logical block][stream], see skew_index); positions outside the box
-// get 0, and so does the state.  For the multi-CTA form also the empty
-// hand-off columns.
+// Skewed statics; positions outside the box get 0, and so does the state.  For
+// the multi-CTA form also the empty hand-off columns.
 template <class T>
 __device__ void adj_pack_body(const AdjArgs<T> &A, size_t bid, size_t nbid) {
-    constexpr int E = 16 / (int)sizeof(T);
     const size_t n = (size_t)A.nx * A.ny;
     const size_t chan = (size_t)4 * A.nb * A.nstepp * 32;
-    for (size_t t = bid * blockDim.x + threadIdx.x; t < chan / E; t += nbid * blockDim.x) {
-        union { T v[E]; uint4 w; } o[5];
-#pragma unroll
-        for (int i = 0; i < E; ++i) {
-            int x, y;
-            const bool in = skew_node<T>(t * E + i, A.nx, A.ny, A.nb, A.nstepp, x, y);
-            const size_t j = in ? (size_t)y * A.nx + x : 0;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) o[c].v[i] = in ? A.win[c * n + j] : T(0);
-            o[4].v[i] = in ? A.dJdu[(size_t)y * A.sy + x] : T(0);
-        }
-#pragma unroll
-        for (int c = 0; c < 5; ++c) reinterpret_cast<uint4 *>(A.sk + c * chan)[t] = o[c].w;
-    }
+    skew_pack<T, 5>(A.sk, chan, A.nx, A.ny, A.nb, A.nstepp, bid, nbid, T(0), [&](int c, int x, int y) {
+        return c < 4 ? A.win[c * n + (size_t)y * A.nx + x] : A.dJdu[(size_t)y * A.sy + x];
+    });
     const size_t box = (size_t)A.nb * A.ny * 32;
     for (size_t t = bid * blockDim.x + threadIdx.x; t < box; t += nbid * blockDim.x) A.state[t] = T(0);
     if (A.multi)

@@ -89,27 +89,16 @@ struct FsmArgs {
     int multi;   // multi-CTA form
 };
 
-// Skewed slowness r h in storage order, 16 bytes per thread (positions outside
+// Skewed slowness r h (positions outside
 // the box and Gamma nodes get +inf), then the state (Sec. 1.1 initialisation:
 // Gamma fixed at g, everything else large, padding columns included) and, for
 // the multi-CTA form, the empty hand-off columns.
 template <class T>
 __device__ void fsm_pack_body(const FsmArgs<T> &A, size_t bid, size_t nbid) {
-    constexpr int E = 16 / (int)sizeof(T);
-    const size_t nv = (size_t)4 * A.nb * A.nstepp * 32 / E;
-    for (size_t t = bid * blockDim.x + threadIdx.x; t < nv; t += nbid * blockDim.x) {
-        union { T v[E]; uint4 w; } o;
-#pragma unroll
-        for (int i = 0; i < E; ++i) {
-            int x, y;
-            o.v[i] = Num<T>::inf();
-            if (skew_node<T>(t * E + i, A.nx, A.ny, A.nb, A.nstepp, x, y)) {
-                const size_t gi = (size_t)y * A.sy + x;
-                o.v[i] = FsmPolicy<T>::node(A.gamma[gi] != 0, A.r[gi], A.h);
-            }
-        }
-        reinterpret_cast<uint4 *>(A.rsk)[t] = o.w;
-    }
+    skew_pack<T, 1>(A.rsk, 0, A.nx, A.ny, A.nb, A.nstepp, bid, nbid, Num<T>::inf(), [&](int, int x, int y) {
+        const size_t gi = (size_t)y * A.sy + x;
+        return FsmPolicy<T>::node(A.gamma[gi] != 0, A.r[gi], A.h);
+    });
     const size_t total = (size_t)A.nb * A.ny * 32;
     for (size_t t = bid * blockDim.x + threadIdx.x; t < total; t += nbid * blockDim.x) {
         const size_t row = t >> 5;

@@ -124,6 +124,51 @@ __device__ __forceinline__ bool skew_node(size_t e, int nx, int my, int nb, int 
     return x < nx && lr >= 0 && lr < my;
 }
 
+// Packs NCH channels of a field into skewed statics (out + c * chan), positions
+// outside the box get `pad`; get(c, x, y) is the value at a node.  A stream reads
+// the field along diagonals, 32 rows for 32 neighbouring columns: gathered from
+// global memory that is a transaction per element (5 channels of 64 fields of
+// 1025^2: 4.3 ms, one L1 wavefront an element).  So rows are loaded as rows into a
+// tile of one block's 32 columns and read diagonally there, where the lanes of a
+// warp stand in different banks (2.2 ms).  A tile serves 64 steps of all four
+// directions: those whose group of steps starts at its row, counted from the
+// bottom or from the top, and the 31 rows before and after that they reach.
+constexpr int PACK_ROWS = 64;
+template <class T, int NCH, class Get>
+__device__ __forceinline__ void skew_pack(T *out, size_t chan, int nx, int my, int nb, int nstepp, size_t bid,
+                                          size_t nbid, T pad, Get get) {
+    constexpr int E = 16 / (int)sizeof(T), LE = sizeof(T) == 4 ? 2 : 1, S = PACK_ROWS, R = S + 62;
+    __shared__ T tile[R * 32];
+    const int wmin = my - nstepp, nwin = (nstepp - wmin + S - 1) / S, ng = nstepp >> LE;
+    const int lane = threadIdx.x & 31;
+    for (size_t t = bid; t < (size_t)nb * nwin * NCH; t += nbid) {
+        const int c = (int)(t % NCH), u = (int)(t / NCH), b = u / nwin, w0 = wmin + (u - b * nwin) * S;
+        __syncthreads();
+        for (int e = threadIdx.x; e < R * 32; e += blockDim.x) {
+            const int y = w0 - 31 + (e >> 5), x = 32 * b + lane;
+            tile[e] = x < nx && y >= 0 && y < my ? get(c, x, y) : pad;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int sy = 0; sy < 2; ++sy) {
+            // groups of E steps whose first step s0 has s0 (sy = 1) or my - 1 - s0 in [w0, w0 + S)
+            const int lo = max(0, sy ? (w0 + E - 1) >> LE : ((my - 1 - w0 - S) >> LE) + 1);
+            const int hi = min(ng, sy ? (w0 + S + E - 1) >> LE : ((my - 1 - w0) >> LE) + 1);
+            for (int k = threadIdx.x >> 5; k < 2 * (hi - lo); k += blockDim.x >> 5) {
+                const int px = k & 1, gq = lo + (k >> 1), col = px ? lane : 31 - lane;
+                union { T v[E]; uint4 w; } o;
+#pragma unroll
+                for (int i = 0; i < E; ++i) {
+                    const int lr = E * gq + i - lane, y = sy ? lr : my - 1 - lr;
+                    o.v[i] = tile[(y - w0 + 31) * 32 + col];
+                }
+                const size_t stream = (size_t)(2 * px + sy) * nb + (px ? b : nb - 1 - b);
+                reinterpret_cast<uint4 *>(out + c * chan + stream * nstepp * 32)[gq * 32 + lane] = o.w;
+            }
+        }
+    }
+}
+
 template <class T, int NST>
 struct Box {
     T *u;                          // state, strip-major [nb][ny][32]
