@@ -46,13 +46,15 @@ __host__ __device__ inline size_t box2_smem_bytes(int nx, int ny) {
 // 32.2, 65^2 8.8 / 32.6 against 16.3 / 66.7, 97^2 14.8 / 124 against 21.0 / 120,
 // 129^2 (K = 5) 23 / 394 against 27 / 200.  FP64, where one warp has a quarter
 // of an SM's FP64 rate (64 cycles an operation) and the engine's warps have all
-// of it: 33^2 59 against 63, 65^2 173 against 92.  Two boxes fit an SM.
+// of it, whole grids: 17^2 266 us against 423, 32^2 520 / 675, 33^2 1078 / 1194,
+// but 41^2 1386 / 1294, 64^2 3616 / 2644: up to 36 columns.  `most`: shared memory
+// that leaves room for two boxes on an SM; a single box may take more.
 template <class T>
 __host__ __device__ constexpr int box2_kmax() { return sizeof(T) == 4 ? 4 : 2; }
 template <class T>
-__host__ __device__ inline int box2_use(int nx, int ny) {
+__host__ __device__ inline int box2_use(int nx, int ny, size_t most = 100 << 10) {
     const int k = box2_k(nx);
-    return k <= box2_kmax<T>() && box2_smem_bytes<T>(nx, ny) <= (size_t)(100 << 10) ? k : 0;
+    return k <= box2_kmax<T>() && (sizeof(T) == 4 || nx <= 36) && box2_smem_bytes<T>(nx, ny) <= most ? k : 0;
 }
 
 // Where the nodes of a box stand in its two shared arrays.

@@ -10,6 +10,7 @@
 #include <cstring>
 
 #include "common.cuh"
+#include "box2.cuh"
 #include "engine.cuh"
 #include "host_util.h"
 #include "prof.h"
@@ -201,6 +202,58 @@ __global__ void k_fsm_unpack(FsmArgs<T> A, eik_fsm_stats *out) {
     fsm_unpack_body(A, out, blockIdx.x, gridDim.x);
 }
 
+// A small grid from the caller's arrays to u in one launch, swept by one warp in
+// shared memory (box2.cuh).  97 x 101 FP32, 24 sweeps: 0.45 ms a call, packed and
+// by the engine 0.67 ms.
+template <int K, class T>
+__device__ __forceinline__ void fsm_box_body(const FsmArgs<T> &A, char *smem, eik_fsm_stats *out) {
+    const Box2<K> B(A.nx, A.ny);
+    T *const su = reinterpret_cast<T *>(smem), *const sr = su + B.cells();
+    for (int i = threadIdx.x; i < 2 * B.cells(); i += blockDim.x) su[i] = Num<T>::inf();
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int y = warp; y < A.ny; y += nw)
+        for (int x = lane; x < A.nx; x += 32) {
+            const size_t gi = (size_t)y * A.sy + x;
+            const bool gam = A.gamma[gi] != 0;
+            const T rv = A.r[gi], gv = A.g[gi];
+            const int q = B.at(x, y);
+            sr[q] = FsmPolicy<T>::node(gam, rv, A.h);
+            if (gam) su[q] = gv;
+        }
+    __syncthreads();
+    if (warp == 0) {
+        long long sweeps;
+        bool conv;
+        box2_sweeps<K, T>(B, (unsigned)__cvta_generic_to_shared(su), (unsigned)__cvta_generic_to_shared(sr),
+                          A.max_sweeps, sweeps, conv);
+        if (out && lane == 0) {
+            out->sweeps = sweeps;
+            out->converged = conv ? 1 : 0;
+            out->error = DEV_OK;
+            out->updates = sweeps * A.nx * A.ny;
+            out->launches = A.launches;
+        }
+    }
+    __syncthreads();
+    for (int y = warp; y < A.ny; y += nw)
+        for (int x = lane; x < A.nx; x += 32) A.u[(size_t)y * A.sy + x] = su[B.at(x, y)];
+}
+
+constexpr int FSM_BOX_THREADS = 512;  // for the copies in and out
+
+template <int K, class T>
+__global__ void __launch_bounds__(FSM_BOX_THREADS) k_fsm_box(FsmArgs<T> A, eik_fsm_stats *out) {
+    extern __shared__ __align__(16) char smem[];
+    fsm_box_body<K, T>(A, smem, out);
+}
+template <class T>
+constexpr void (*fsm_box_kernel(int k))(FsmArgs<T>, eik_fsm_stats *) {
+    if constexpr (box2_kmax<T>() > 2)
+        if (k > 2) return k == 3 ? k_fsm_box<3, T> : k_fsm_box<4, T>;
+    return k == 1 ? k_fsm_box<1, T> : k_fsm_box<2, T>;
+}
+
 // Widest grid (32-column blocks) swept by one CTA.  Above it the blocks' warps
 // share too few schedulers and spreading them over CTAs wins in spite of the
 // slower hand-off (FP32 us a sweep, one CTA / several: 257^2 50.6 / 51.2,
@@ -266,8 +319,16 @@ static int fsm_run(const eik_grid *grid, const FsmPlan &P, const void *r, const 
     A.h = (T)grid->h;
     A.max_sweeps = max_sweeps;
     fsm_layout<T>(P, &A, ws);
-    A.launches = 3;
     int rc;
+    // one problem, one CTA: it may take most of an SM's shared memory
+    if (const int k = box2_use<T>(P.nx, P.ny, 200 << 10)) {
+        A.launches = 1;
+        const size_t smem = box2_smem_bytes<T>(P.nx, P.ny);
+        void (*const kernel)(FsmArgs<T>, eik_fsm_stats *) = fsm_box_kernel<T>(k);
+        if ((rc = cuda_check(set_dyn_smem(kernel, (int)smem), "smem attr"))) return rc;
+        EIK_LAUNCH("fsm_sweeps", s, kernel<<<1, FSM_BOX_THREADS, smem, s>>>(A, stats));
+        return cuda_check(cudaGetLastError(), "fsm launch");
+    }
     int dev, optin = 0, nsm = 0;
     if ((rc = cuda_check(cudaGetDevice(&dev), "cudaGetDevice"))) return rc;
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -371,6 +432,18 @@ __global__ void k_fsmm_unpack(FsmMany<T> M, eik_fsm_stats *out) {
     fsm_unpack_body(fsm_prob(M, blockIdx.y), out ? out + blockIdx.y : nullptr, blockIdx.x, gridDim.x);
 }
 
+template <int K, class T>
+__global__ void __launch_bounds__(FSM_BOX_THREADS) k_fsmm_box(FsmMany<T> M, eik_fsm_stats *out) {
+    extern __shared__ __align__(16) char smem[];
+    fsm_box_body<K, T>(fsm_prob(M, blockIdx.x), smem, out ? out + blockIdx.x : nullptr);
+}
+template <class T>
+constexpr void (*fsmm_box_kernel(int k))(FsmMany<T>, eik_fsm_stats *) {
+    if constexpr (box2_kmax<T>() > 2)
+        if (k > 2) return k == 3 ? k_fsmm_box<3, T> : k_fsmm_box<4, T>;
+    return k == 1 ? k_fsmm_box<1, T> : k_fsmm_box<2, T>;
+}
+
 struct FsmManyPlan {
     FsmPlan P;
     size_t tab_bytes, per, bytes;
@@ -425,9 +498,14 @@ static int fsm_many_run(const eik_grid *grid, const FsmManyPlan &MP, int nprob, 
     cudaFuncAttributes fa;
     if ((rc = cuda_check(cudaFuncGetAttributes(&fa, k_fsmm_run<T>), "func attr"))) return rc;
     const bool single = (int)P.smem <= optin && P.nb <= 32 && regs_fit(fa, P.nb);
+    const int box_k = box2_use<T>(P.nx, P.ny);
+    const size_t box_smem = box2_smem_bytes<T>(P.nx, P.ny);
     const int nblk = (P.nb + P.wpc - 1) / P.wpc;
     int group = nprob;  // problems per cooperative launch
-    if (!single) {
+    if (box_k) {
+        if ((rc = cuda_check(set_dyn_smem(fsmm_box_kernel<T>(box_k), (int)box_smem), "smem attr")))
+            return rc;
+    } else if (!single) {
         if ((rc = cuda_check(set_dyn_smem(k_fsmm_run_global<T>, (int)P.gsmem), "smem attr")))
             return rc;
         int per_sm = 0;
@@ -452,6 +530,11 @@ static int fsm_many_run(const eik_grid *grid, const FsmManyPlan &MP, int nprob, 
     }
     int nl = upload_ptrs(const_cast<const void **>(M.tab), tab.data(), 3 * nprob, s);
     if (nl < 0) return nl;
+    if (box_k) {
+        A.launches = nl + 1;
+        EIK_LAUNCH("fsm_sweeps", s, fsmm_box_kernel<T>(box_k)<<<nprob, FSM_BOX_THREADS, box_smem, s>>>(M, stats));
+        return cuda_check(cudaGetLastError(), "fsm launch");
+    }
     const int ngroups = (nprob + group - 1) / group;
     nl += 2 + (single ? 1 : 1 + ngroups);
     A.launches = nl;

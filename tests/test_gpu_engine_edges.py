@@ -50,7 +50,7 @@ def test_ranges(gpu, scale, g0):
 
 # Small subdomains, which one warp sweeps with K columns a lane: widths around the 32 K edges, heights from the
 # smallest to the largest that the form takes, and the first ones that go to the engine (FP32: 128 columns by 99
-# rows; FP64: 64 columns).
+# rows; FP64: 36 columns).
 @pytest.mark.parametrize("tiles,cells,c", [((1, 1), (2, 2), 1), ((3, 2), (2, 6), 2), ((2, 2), (30, 4), 2), ((2, 1), (31, 31), 31),
                                            ((1, 2), (32, 40), 4), ((2, 2), (62, 2), 2), ((1, 2), (63, 63), 21),
                                            ((2, 2), (64, 8), 8)])
@@ -75,3 +75,23 @@ def test_small_boxes_f32(gpu, nx, ny, c):
     off = (np.arange(ny)[:, None] % c != 0) & (np.arange(nx)[None, :] % c != 0)
     np.testing.assert_array_equal(u.cpu().numpy()[off], u_ref[off])
     assert st["fsm_sweeps_max"] == st_ref["sweeps"]
+
+
+# plain sweeping of a small grid takes the one-warp form up to 128 (FP64: 36) columns while the box fits an SM; one by
+# itself and several in a call, against the same nodes inside a grid too wide for it: a strip of Gamma nodes at +inf
+# beside them changes nothing
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("nx,ny", [(2, 2), (3, 200), (32, 33), (33, 17), (64, 190), (65, 40), (96, 31), (97, 101), (128, 190),
+                                   (128, 205)])
+def test_small_grids(gpu, nx, ny, dtype):
+    r, gamma, g = _problem((ny, nx), 3 * nx + ny, g0=-0.5 if nx == 33 else 0.0)
+    wide = [np.concatenate([a, np.full((ny, 140), v, a.dtype)], 1) for a, v in ((r, 1.0), (gamma, 1), (g, np.inf))]
+    u_ref, st_ref = _fsm(gpu, *wide, 0.05, dtype)
+    u, st = _fsm(gpu, r, gamma, g, 0.05, dtype)
+    np.testing.assert_array_equal(u, u_ref[:, :nx])
+    assert st["sweeps"] == st_ref["sweeps"]
+    R = torch.from_numpy(r).to(DEV, dtype)
+    gs = [torch.from_numpy(gamma).to(DEV)] * 3
+    us, sts = gpu.fsm_many(R, gs, [torch.from_numpy(g + k).to(DEV, dtype) for k in range(3)], 0.05)
+    np.testing.assert_array_equal(us[0].cpu().numpy(), u)
+    assert sts[0]["sweeps"] == st["sweeps"] and all(s["converged"] == 1 for s in sts)
