@@ -3,7 +3,8 @@
 //
 // Per parareal iteration k the device runs, on one stream:
 //   k_fine   one CTA per subdomain: Step 2 boundary data from (U, W), Step 3
-//            FSM sweeps by the warp-systolic engine, then the Alg. 3 winds of
+//            FSM sweeps by the warp-systolic engine (small boxes: k_fine_box,
+//            by one warp in shared memory), then the Alg. 3 winds of
 //            the converged state at the subdomain's coarse-set nodes (written
 //            as per-subdomain copies) and the fine values of interior nodes;
 //   k_alg4   one thread per coarse-set node: Alg. 4 choice among the copies

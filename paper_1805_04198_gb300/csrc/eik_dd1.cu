@@ -8,13 +8,13 @@
 // lanes each): the 1-D FSM of Sec. 1.1 (Steps 2-3) is a chain of dependent
 // updates, bound by the latency of one FP64 addition and comparison per node
 // where the wave passes; what it does not change is checked by all eight lanes
-// at once (1024 subintervals of 1001 FP64 nodes, two iterations: 1.17 ms; one thread
-// per subinterval, comparisons on the FP64 pipe: 6.5 ms).  CTA 0 holds the coarse state (U, the new U, u^k,
-// C_H(U^k), the winds W^k and w^k, the fixed-node mask) in shared memory and
-// runs the coarse work between two grid barriers: the Step 3 choice at the
-// coarse nodes (its threads), then one warp for the serial part (Step 1's
-// coarse FSM, Step 4's weighted Gauss-Seidel sweeps, the causal sweep, the
-// update size), in the same form.  U and W are published to global
+// at once (1024 subintervals of 1001 FP64 nodes, two iterations: 1.17 ms; one
+// thread per subinterval, comparisons on the FP64 pipe: 6.5 ms).  CTA 0 holds the
+// coarse state (U, the new U, u^k, C_H(U^k), the winds W^k and w^k, the fixed-node
+// mask) in shared memory and runs the coarse work between two grid barriers: the
+// Step 3 choice at the coarse nodes (its threads), then one warp for the serial
+// part (Step 1's coarse FSM, Step 4's weighted Gauss-Seidel sweeps, the causal
+// sweep, the update size), in the same form.  U and W are published to global
 // memory for the next fine phase; the subintervals' end copies come back through
 // global memory.
 // Every grid barrier is a bounded wait: on expiry the kernel records
