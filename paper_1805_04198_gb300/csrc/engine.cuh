@@ -40,11 +40,11 @@
 //
 // What bounds it: the chain of one step (shuffle, two differences, square
 // root, select, minimum), NX + NY of them per sweep, not memory; two boxes of
-// nine warps on an SM are bound by issue.  257^2 FP32 in one CTA 51 us a sweep (85
-// with flags and fences, re-read rows and tests in the step), FP64 308 us; a
-// full 4097^2 FP32 grid 0.97 ms a sweep (2.06).  The sweep direction is a run-time
-// value (one copy of the step code for all four orderings); policies that do not
-// distinguish the sides of an axis (P::SYM) are given the two axis minima.
+// nine warps on an SM issue in two of three cycles.  257^2 FP32 in one CTA 51 us
+// a sweep (85 with flags and fences, re-read rows and tests in the step), FP64 308
+// us; a full 4097^2 FP32 grid 0.97 ms a sweep (2.06).  The sweep direction is a
+// run-time value (one copy of the step code for all four orderings); policies that
+// do not distinguish the sides of an axis (P::SYM) are given the two axis minima.
 //
 // Storage of the state u: strip-major [block][row][32] (row = physical y,
 // 32 = physical x within the block), padded to a whole number of blocks with
