@@ -283,6 +283,16 @@ __device__ __forceinline__ void kb_fine_body(const DDArgs<T> &A, char *smem, int
     k_fine_body<T>(A, smem, tile);
 }
 EIK_BATCH_PAIR(kb_fine, kb_fine_body, 112, 168)
+// The same for FP32 boxes of 17 to 20 blocks: five warps on a scheduler have 102
+// registers a thread, so at kb_fine_f32's 112 the launch has no room (16 warps and
+// fewer: four on a scheduler).  At 96 a batch of 1025^2 and 513^2 solves in
+// subdomains of 513^2 and 257^2, seven passes, runs in 145 ms.
+__global__ void __maxnreg__(96) kb_fine_wide_f32(const DDArgs<float> *__restrict__ args, ItemList L) {
+    extern __shared__ __align__(16) char smem[];
+    class_begin();
+    for_items(L, [&](int p, int local) { kb_fine_body<float>(args[p], smem, local); });
+    class_end();
+}
 template <int K, class T>
 __global__ void __launch_bounds__(BOX2_THREADS) kb_fine_box(const DDArgs<T> *__restrict__ args, ItemList L) {
     extern __shared__ __align__(16) char smem[];
@@ -307,12 +317,14 @@ template <> struct BatchKernels<float> {
     static constexpr void (*step4)(const DDArgs<float> *, ItemList) = kb_step4_f32;
     static constexpr void (*step4a)(const DDArgs<float> *, ItemList) = kb_step4a_f32;
     static constexpr void (*fine)(const DDArgs<float> *, ItemList) = kb_fine_f32;
+    static constexpr void (*fine_wide)(const DDArgs<float> *, ItemList) = kb_fine_wide_f32;
 };
 template <> struct BatchKernels<double> {
     static constexpr void (*step1)(const DDArgs<double> *, ItemList) = kb_step1_f64;
     static constexpr void (*step4)(const DDArgs<double> *, ItemList) = kb_step4_f64;
     static constexpr void (*step4a)(const DDArgs<double> *, ItemList) = kb_step4a_f64;
     static constexpr void (*fine)(const DDArgs<double> *, ItemList) = kb_fine_f64;
+    static constexpr void (*fine_wide)(const DDArgs<double> *, ItemList) = kb_fine_f64;  // (at most nine blocks)
 };
 
 // --------------------------------------------------------------------------
@@ -554,7 +566,12 @@ static int batch_run(int nprob, const eik_grid *grids, const void *const *r, con
         set_error("shared memory need (%zu, %zu) exceeds the device limit %d", limit_fine, limit_grid, smem_optin);
         return EIK_EUNSUPPORTED;
     }
-    auto finek = [](const BoxClass &c) { return c.box_k ? fine_box_kernel<T>(c.box_k) : BatchKernels<T>::fine; };
+    cudaFuncAttributes fa;
+    if ((rc = cuda_check(cudaFuncGetAttributes(&fa, BatchKernels<T>::fine), "func attr"))) return rc;
+    auto finek = [&](const BoxClass &c) {
+        if (c.box_k) return fine_box_kernel<T>(c.box_k);
+        return regs_fit(fa, c.nw) ? BatchKernels<T>::fine : BatchKernels<T>::fine_wide;
+    };
     for (auto it = B.fine.begin(); it != B.fine.end(); ++it) {
         size_t need = it->smem;
         for (auto &c : B.fine)

@@ -252,3 +252,21 @@ def test_batched_adaptive_weight_mixed(gpu, dtype):
             assert torch.equal(B.u[i], u1), i
             for key in ("iters", "converged", "fine_updates", "coarse_updates", "coarse_cap_hits"):
                 assert stats[i][key] == s1[key], (i, key)
+
+
+def test_batched_wide_subdomains(gpu):
+    """FP32 subdomains of 513, 577 and 609 columns, the widest an SM's shared memory holds (17 to 20 warps a box), in
+    one batch with a narrow one: bitwise the single solves."""
+    probs = [_problem(shape, tiles, c, 0.0, 2, seed=i)
+             for i, (shape, tiles, c) in enumerate([((513, 1025), (2, 1), 16), ((161, 577), (1, 1), 32),
+                                                    ((17, 609), (1, 1), 16), ((257, 257), (4, 4), 8)])]
+    for p in probs:
+        p["gamma"] = _t(p["gamma"], torch.uint8)
+        p["r"], p["g"] = _t(p["r"].astype(np.float32), torch.float32), _t(p["g"], torch.float32)
+    B = gpu.DDBatch(probs)
+    B.run()
+    stats = B.stats()
+    for i, p in enumerate(probs):
+        u, st = _single(gpu, p)
+        assert torch.equal(B.u[i], u), i
+        assert stats[i]["error"] == 0 and stats[i]["iters"] == st["iters"], i
