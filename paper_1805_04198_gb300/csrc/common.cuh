@@ -91,9 +91,10 @@ __device__ __forceinline__ Root64 root_start(double x) {
     R.unsure = ((f + 3) & 4095) <= 4 || (unsigned)(e + 900) > 1800u;
     return R;
 }
-__device__ __forceinline__ void root_decide(Root64 &R) {
+// `clamp`: the root of max(x, 0), 0 where x is NaN.
+__device__ __forceinline__ void root_decide(Root64 &R, bool clamp = false) {
     if ((unsigned)((__double2hiint(R.x) >> 20) - 1023 + 900) > 1800u) {
-        R.out = __double_as_longlong(__dsqrt_rn(R.x));
+        R.out = __double_as_longlong(__dsqrt_rn(clamp ? fmax(R.x, 0.0) : R.x));
         R.qe = 0;
         return;
     }
@@ -115,6 +116,7 @@ __device__ __forceinline__ double sqrt_rn64(double x) {
 template <> struct Num<float> {
     static __device__ __forceinline__ bool lt(float a, float b) { return a < b; }
     static __device__ __forceinline__ bool le(float a, float b) { return a <= b; }
+    static __device__ __forceinline__ bool lowers(float ut, float self) { return ut < self; }
     static __device__ __forceinline__ float mn(float a, float b) { return fminf(a, b); }
     static __device__ __forceinline__ bool below(float d, float rh) { return fabsf(d) < rh; }
     static __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
@@ -138,6 +140,13 @@ template <> struct Num<double> {
     // (operands are never NaN)
     static __device__ __forceinline__ bool lt(double a, double b) { return key(a) < key(b); }
     static __device__ __forceinline__ bool le(double a, double b) { return key(a) <= key(b); }
+    // ut < self, false where ut is NaN (the keys of NaNs with the sign set, which
+    // arithmetic gives, are below that of -inf).  For the three-term branch; the
+    // two-term one gives no NaN, and the test would cost a small box 4%.
+    static __device__ __forceinline__ bool lowers(double ut, double self) {
+        const long long k = key(ut);
+        return k < key(self) && (int)(k >> 32) >= (int)0x800fffff;
+    }
     static __device__ __forceinline__ double mn(double a, double b) { return lt(a, b) ? a : b; }
     // |d| < rh for rh >= 0, false where d is NaN
     static __device__ __forceinline__ bool below(double d, double rh) { return mag(d) < bits64(rh); }
@@ -165,9 +174,9 @@ constexpr uint8_t WIND_ECHO = 0x80;
 
 // Value of the local solve from the axis minima a, b: the two-term branch
 // (a + b + sqrt(2 r^2 h^2 - (a-b)^2)) / 2 where |a - b| < r h, else the smaller
-// one plus r h.  The discriminant needs no clamp: where the two-term branch is
-// taken it is at least (r h)^2; where it is negative or NaN its root is not
-// selected.
+// one plus r h.  The discriminant needs no clamp while (r h)^2 is finite: where
+// the two-term branch is taken it is at least (r h)^2; elsewhere its root is not
+// selected.  Where both squares overflow it is NaN, which counts as 0 in FP64.
 __device__ __forceinline__ float solve2(float a, float b, float rh, bool &two) {
     using N = Num<float>;
     const float d = N::sub(a, b);
@@ -194,9 +203,12 @@ __device__ __forceinline__ Solve64 solve2_start(double a, double b, double rh) {
     Solve64 S;
     const double d = N::sub(a, b);
     S.two = N::below(d, rh) && __double2hiint(rh) < 0x7ff00000;
-    // 2 r h by its exponent (exact; where r h is subnormal its square is 0 in any
-    // case).  Not 2 (r h)^2: that loses the bits of a square just below the normal range.
-    const double rh2 = __hiloint2double(__double2hiint(rh) + (1 << 20), __double2loint(rh));
+    // 2 r h by its exponent (exact, +inf above the range; where r h is subnormal
+    // its square is 0 in any case).  Not 2 (r h)^2: that loses the bits of a square
+    // just below the normal range.
+    const int rhi = __double2hiint(rh);
+    const bool top = rhi >= 0x7fe00000;
+    const double rh2 = __hiloint2double(top ? 0x7ff00000 : rhi + (1 << 20), top ? 0 : __double2loint(rh));
     const double disc = N::sub(N::mul(rh2, rh), N::mul(d, d));
     S.root = root_start(S.two ? disc : 1.0);
     S.ab = N::add(a, b);
@@ -215,7 +227,7 @@ __device__ __forceinline__ double solve2_end(const Solve64 &S) {
 }
 __device__ __forceinline__ double solve2(double a, double b, double rh, bool &two) {
     Solve64 S = solve2_start(a, b, rh);
-    if (S.root.unsure) root_decide(S.root);
+    if (S.root.unsure) root_decide(S.root, true);
     two = S.two;
     return solve2_end(S);
 }
@@ -295,7 +307,7 @@ __device__ __forceinline__ T local_solve3(const T *vm, const T *vp, T rh, uint8_
 
 // x / 3, correctly rounded: the quotient by the rounded reciprocal corrected by
 // its exact residual (Markstein, as above; equal to the division for every
-// finite float but -0).  NaN at +-inf.
+// finite number but -0).  NaN at +-inf.
 __device__ __forceinline__ float div3(float x) {
     const float c = 1.f / 3.f;
     const float q = __fmul_rn(x, c);
@@ -309,8 +321,8 @@ __device__ __forceinline__ double div3(double x) {
 
 // Value of the 3-D local solve from the three axis minima (the same rounded
 // operations as local_solve3 on the sorted values): a sort of minima and maxima,
-// no winds.  r h = +inf (fixed nodes) gives +inf or, in FP32, NaN: neither is
-// below any value.
+// no winds.  r h = +inf (fixed nodes) gives +inf or, in FP32, NaN, and squares
+// that overflow may give NaN: neither lowers any value.
 __device__ __forceinline__ float solve3(float m0, float m1, float m2, float rh) {
     using N = Num<float>;
     const float lo = fminf(m0, m1), hi = fmaxf(m0, m1);
@@ -342,7 +354,7 @@ __device__ __forceinline__ double solve3(double m0, double m1, double m2, double
         const double sd = N::add(d1, d2);
         double disc3 = N::sub(N::mul(sd, sd), N::mul(3.0, N::sub(N::add(N::mul(d1, d1), N::mul(d2, d2)), N::mul(rh, rh))));
         if (disc3 < 0.0) disc3 = 0.0;
-        u = N::add(v0, div3(N::add(sd, disc3 > 0.0 ? sqrt_rn64(disc3) : 0.0)));
+        u = N::add(v0, div3(N::add(sd, sqrt_rn64(disc3))));
     }
     return u;
 }

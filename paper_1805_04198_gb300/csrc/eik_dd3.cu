@@ -383,7 +383,7 @@ struct Fsm3Update {
     __device__ __forceinline__ T apply(T self, const T *vm, const T *vp, T rh, bool &changed) const {
         using N = Num<T>;
         const T ut = solve3(N::mn(vm[0], vp[0]), N::mn(vm[1], vp[1]), N::mn(vm[2], vp[2]), rh);
-        changed = N::lt(ut, self);
+        changed = N::lowers(ut, self);
         return changed ? ut : self;
     }
 };

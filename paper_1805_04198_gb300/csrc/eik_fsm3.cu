@@ -388,7 +388,7 @@ __device__ int fsm3_tile_sweep(const Fsm3Args<T> &A, int b, int k, long long wli
             if (j == 3) yp = y[s];
             const bool on = ok(m0 + s);
             const T ut = solve3(N::mn(xm, xp), N::mn(ym, yp), N::mn(last, nxt), r[s]);
-            const bool ch = on && N::lt(ut, cur);
+            const bool ch = on && N::lowers(ut, cur);
             const T v = ch ? ut : cur;
             p3_sthand(outx && on, ox0 + s, v);
             p3_sthand(outy && on, oy0 + s, v);

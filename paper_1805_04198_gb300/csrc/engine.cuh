@@ -388,7 +388,7 @@ struct FsmPolicy {
         if (unsure) {
 #pragma unroll
             for (int j = 0; j < K; ++j)
-                if (S[j].root.unsure) root_decide(S[j].root);
+                if (S[j].root.unsure) root_decide(S[j].root, true);
         }
 #pragma unroll
         for (int j = 0; j < K; ++j) {

@@ -1,0 +1,76 @@
+"""Values at the ends of the FP64 range, against plain serial sweeps of the same closed form in numpy.
+
+Where (r h)^2 overflows the discriminant of the two-term branch is +inf or, if the difference squared overflows too,
+NaN, which counts as 0; a NaN of the three-term branch leaves the node as it is."""
+import itertools
+
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _solve(mins, rh):
+    """The Godunov local solve from the minima of the two or three axes."""
+    a = sorted(mins)
+    d = a[0] - a[1]
+    if not abs(d) < rh:
+        return a[0] + rh
+    u = (a[0] + a[1] + np.sqrt(np.fmax((2.0 * rh) * rh - d * d, 0.0))) * 0.5
+    if len(a) == 3 and u > a[2]:
+        d1, d2 = a[1] - a[0], a[2] - a[0]
+        disc = (d1 + d2) * (d1 + d2) - 3.0 * ((d1 * d1 + d2 * d2) - rh * rh)
+        u = a[0] + ((d1 + d2) + np.sqrt(0.0 if disc < 0.0 else disc)) / 3.0
+    return u
+
+
+def sweeps(r, gamma, g, h, most):
+    """Serial sweeps in the 2^d orderings (the sign of x outermost, -1 first) until one changes nothing, `most` at
+    most."""
+    shape = r.shape
+    u = np.full([s + 2 for s in shape], np.inf)
+    core = tuple(slice(1, s + 1) for s in shape)
+    u[core] = np.where(gamma != 0, g, np.inf)
+    dim = len(shape)
+    for k in range(most):
+        changed = False
+        signs = [(k >> a) & 1 for a in range(dim)]  # of the axes of the array: the last one, x, is the highest bit
+        for at in itertools.product(*(range(s) if up else range(s - 1, -1, -1) for s, up in zip(shape, signs))):
+            if gamma[at]:
+                continue
+            c = tuple(i + 1 for i in at)
+            mins = []
+            for a in range(dim):
+                lo = c[:a] + (c[a] - 1,) + c[a + 1:]
+                hi = c[:a] + (c[a] + 1,) + c[a + 1:]
+                mins.append(np.fmin(u[lo], u[hi]))
+            v = _solve(mins, r[at] * h)
+            if v < u[c]:
+                u[c] = v
+                changed = True
+        if not changed:
+            return u[core], k + 1
+    return u[core], most
+
+
+def _dev(*arrs):
+    return [torch.from_numpy(np.ascontiguousarray(a)).to(DEV) for a in arrs]
+
+
+# one warp, one thread block and several in 2-D, tiles in 3-D
+@pytest.mark.parametrize("shape", [(11, 9), (7, 40), (4, 300), (5, 6, 11)])
+@pytest.mark.parametrize("scale", [1e153, 1e154, 1e155, 1e200, 1e300, 1.2e308])
+def test_squares_above_the_range(gpu, shape, scale):
+    rng = np.random.default_rng(sum(shape))
+    r = scale * rng.choice([1.0, 0.75, 0.5], shape)
+    gamma = np.zeros(shape, np.uint8)
+    gamma[tuple(s // 2 for s in shape)] = gamma[(0,) * len(shape)] = 1
+    g = np.zeros(shape)
+    g[(0,) * len(shape)] = 0.125 * scale
+    with np.errstate(all="ignore"):
+        u_ref, n = sweeps(r, gamma, g, 1.0, 12)
+    u, st = gpu.fsm(*_dev(r, gamma, g), 1.0, max_sweeps=12)
+    np.testing.assert_array_equal(u.cpu().numpy(), u_ref)
+    assert st["sweeps"] == n
