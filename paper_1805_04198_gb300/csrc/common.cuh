@@ -115,10 +115,10 @@ __device__ __forceinline__ double sqrt_rn64(double x) {
 
 template <> struct Num<float> {
     static __device__ __forceinline__ bool lt(float a, float b) { return a < b; }
-    static __device__ __forceinline__ bool le(float a, float b) { return a <= b; }
+    static __device__ __forceinline__ bool below(float a, float b) { return a < b; }
     static __device__ __forceinline__ bool lowers(float ut, float self) { return ut < self; }
     static __device__ __forceinline__ float mn(float a, float b) { return fminf(a, b); }
-    static __device__ __forceinline__ bool below(float d, float rh) { return fabsf(d) < rh; }
+    static __device__ __forceinline__ bool within(float d, float rh) { return fabsf(d) < rh; }
     static __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
     static __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
     static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
@@ -137,9 +137,16 @@ template <> struct Num<float> {
 };
 
 template <> struct Num<double> {
-    // (operands are never NaN)
-    static __device__ __forceinline__ bool lt(double a, double b) { return key(a) < key(b); }
-    static __device__ __forceinline__ bool le(double a, double b) { return key(a) <= key(b); }
+    // a < b as IEEE has it: the two zeros are equal, false where either is NaN.
+    // Where a tie decides something (winds, Alg. 5)
+    static __device__ __forceinline__ bool lt(double a, double b) {
+        constexpr long long top = 0x7ff0000000000000ll;
+        const long long x = key(a) - (bits64(a) >> 63), y = key(b) - (bits64(b) >> 63);
+        return x < y && x >= -top && y <= top;
+    }
+    // a < b by the keys, for the values of a sweep: there a tie of zeros decides
+    // at most the sign of a zero, and one comparison is enough
+    static __device__ __forceinline__ bool below(double a, double b) { return key(a) < key(b); }
     // ut < self, false where ut is NaN (the keys of NaNs with the sign set, which
     // arithmetic gives, are below that of -inf).  For the three-term branch; the
     // two-term one gives no NaN, and the test would cost a small box 4%.
@@ -147,9 +154,9 @@ template <> struct Num<double> {
         const long long k = key(ut);
         return k < key(self) && (int)(k >> 32) >= (int)0x800fffff;
     }
-    static __device__ __forceinline__ double mn(double a, double b) { return lt(a, b) ? a : b; }
+    static __device__ __forceinline__ double mn(double a, double b) { return below(a, b) ? a : b; }
     // |d| < rh for rh >= 0, false where d is NaN
-    static __device__ __forceinline__ bool below(double d, double rh) { return mag(d) < bits64(rh); }
+    static __device__ __forceinline__ bool within(double d, double rh) { return mag(d) < bits64(rh); }
     static __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
     static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
     static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
@@ -202,7 +209,7 @@ __device__ __forceinline__ Solve64 solve2_start(double a, double b, double rh) {
     using N = Num<double>;
     Solve64 S;
     const double d = N::sub(a, b);
-    S.two = N::below(d, rh) && __double2hiint(rh) < 0x7ff00000;
+    S.two = N::within(d, rh) && __double2hiint(rh) < 0x7ff00000;
     // 2 r h by its exponent (exact, +inf above the range; where r h is subnormal
     // its square is 0 in any case).  Not 2 (r h)^2: that loses the bits of a square
     // just below the normal range.
@@ -341,11 +348,11 @@ __device__ __forceinline__ float solve3(float m0, float m1, float m2, float rh) 
 }
 __device__ __forceinline__ double solve3(double m0, double m1, double m2, double rh) {
     using N = Num<double>;
-    const bool s01 = N::lt(m1, m0);
+    const bool s01 = N::below(m1, m0);
     const double lo = s01 ? m1 : m0, hi = s01 ? m0 : m1;
-    const bool s2 = N::lt(m2, lo);
+    const bool s2 = N::below(m2, lo);
     const double v0 = s2 ? m2 : lo, t = s2 ? lo : m2;
-    const bool s3 = N::lt(t, hi);
+    const bool s3 = N::below(t, hi);
     const double v1 = s3 ? t : hi, v2 = s3 ? hi : t;
     bool two;
     double u = solve2(v0, v1, rh, two);

@@ -420,7 +420,7 @@ __device__ __forceinline__ bool sub_sweep(const Line<T, SM> &L, bool on) {
                     if (i + k > 0) t = Num<T>::add(t, __shfl_sync(FULL, rh[i], k, G));
                     if (lane == k) v[i] = t;
                 }
-                followed &= (i == 0 && lane == 0) | (i * G + lane >= left) | Num<T>::lt(v[i], rest[i]);
+                followed &= (i == 0 && lane == 0) | (i * G + lane >= left) | Num<T>::below(v[i], rest[i]);
             }
         }
         if (__any_sync(FULL, !kept && !followed)) {

@@ -365,7 +365,7 @@ struct FsmPolicy {
     }
     __device__ __forceinline__ T update(T self, T a, T b, T rh, bool &changed) const {
         const T ut = local_solve2_min(a, b, rh);
-        changed = Num<T>::lt(ut, self);
+        changed = Num<T>::below(ut, self);
         return changed ? ut : self;
     }
     // K independent nodes; their FP64 roots run together
@@ -393,7 +393,7 @@ struct FsmPolicy {
 #pragma unroll
         for (int j = 0; j < K; ++j) {
             const double ut = solve2_end(S[j]);
-            changed[j] = Num<double>::lt(ut, self[j]);
+            changed[j] = Num<double>::below(ut, self[j]);
             v[j] = changed[j] ? ut : self[j];
         }
     }

@@ -1,12 +1,14 @@
-"""Values at the ends of the FP64 range, against plain serial sweeps of the same closed form in numpy.
+"""Values at the ends of the FP64 range and signs of zero.
 
-Where (r h)^2 overflows the discriminant of the two-term branch is +inf or, if the difference squared overflows too,
+Against plain serial sweeps of the same closed form in numpy: where (r h)^2 overflows the discriminant of the two-term branch is +inf or, if the difference squared overflows too,
 NaN, which counts as 0; a NaN of the three-term branch leaves the node as it is."""
 import itertools
 
 import numpy as np
 import pytest
 import torch
+
+import oracle as O
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -74,3 +76,29 @@ def test_squares_above_the_range(gpu, shape, scale):
     u, st = gpu.fsm(*_dev(r, gamma, g), 1.0, max_sweeps=12)
     np.testing.assert_array_equal(u.cpu().numpy(), u_ref)
     assert st["sweeps"] == n
+
+
+# a node between two Gamma nodes at -0 and +0: a tie, which goes to the plus side
+@pytest.mark.parametrize("tiles,cells,c", [((2, 2), 16, 8), ((1, 2), 60, 10), ((2, 2, 2), 8, 4)])
+@pytest.mark.parametrize("z", [0.0, -0.0])
+@pytest.mark.parametrize("step", ["fine", "coarse"])
+def test_signs_of_zero(gpu, tiles, cells, c, z, step):
+    shape = tuple(t * cells + 1 for t in reversed(tiles))
+    rng = np.random.default_rng(len(shape) + cells)
+    r = rng.uniform(0.5, 2.0, shape)
+    gamma, g = np.zeros(shape, np.uint8), np.zeros(shape)
+    w = 1 if step == "fine" else c  # neighbours of coarse node (c, c) on the fine grid or on its coarse grid
+    for x, v in ((c - w, z), (c + w, -z)):
+        at = (c,) * (len(shape) - 1) + (x,)
+        gamma[at], g[at] = 1, v
+    kw = dict(theta=0.2, max_iter=3, tol=0.0, max_coarse_sweeps=8)
+    u_ref, s_ref, _, U_ref = O.dd(r, gamma, g, 0.05, tiles, c, return_coarse=True, **kw)
+    u, st, *coarse = gpu.dd_solve(*_dev(r, gamma, g), 0.05, tiles, c, return_coarse=len(shape) == 2, **kw)
+    np.testing.assert_array_equal(u.cpu().numpy(), u_ref)
+    assert st["iters"] == s_ref["iters"]
+    if coarse:
+        U = coarse[0].cpu().numpy()
+        on = ~np.isnan(U)
+        np.testing.assert_array_equal(U[on], U_ref[on])
+        if step == "fine":  # the x component of its wind: from the plus side
+            assert int(coarse[1][c, c]) & 3 == 0
