@@ -13,9 +13,9 @@
 //    ahead of it.
 // A sweep takes NX + NY steps, whatever K is; the K local solves of a step are
 // independent and hide each other's latency, and a second sweep starts at once.
-// Rows outside the box are read as the guard rows -1 and NY, which stay +inf like
-// the padding columns: u~ is then +inf, never below the value, and nothing is
-// stored, so rows and columns need no tests.
+// Rows outside the box are read as the guard rows -1 and NY, which like the
+// padding columns stay +inf, their r h being NaN: u~ is never below the value and
+// nothing is stored, so rows and columns need no tests.
 //
 // Shared memory: u and r h, [row -1 .. NY][P]; column K l + j stands at j * NL + l,
 // so that neighbouring lanes, K rows and one column apart, are an odd number of
@@ -70,6 +70,14 @@ struct Box2 {
         return (y + 1) * p + (x - l * K) * nl + l;
     }
     __device__ __forceinline__ int cells() const { return (ny + 2) * p; }
+    // u +inf and r h NaN everywhere (all threads; a barrier must follow)
+    template <class T>
+    __device__ __forceinline__ void clear(T *su, T *sr) const {
+        for (int i = threadIdx.x; i < cells(); i += blockDim.x) {
+            su[i] = Num<T>::inf();
+            sr[i] = Num<T>::nan();
+        }
+    }
 };
 
 // Sweeps until one changes nothing or max_sweeps ran; called by one whole warp,

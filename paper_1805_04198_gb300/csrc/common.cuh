@@ -125,6 +125,7 @@ template <> struct Num<float> {
     static __device__ __forceinline__ float sqrt_(float a) { return __fsqrt_rn(a); }
     static __device__ __forceinline__ float div(float a, float b) { return __fdiv_rn(a, b); }
     static __device__ __forceinline__ float inf() { return __int_as_float(0x7f800000); }
+    static __device__ __forceinline__ float nan() { return __int_as_float(0x7fffffff); }
     // Square root used inside the local solve.  FP32 storage carries a 1e-5
     // accuracy budget, so the single-instruction hardware approximation
     // (relative error ~1e-7, applied only to the increment of the two-term
@@ -163,8 +164,20 @@ template <> struct Num<double> {
     static __device__ __forceinline__ double sqrt_(double a) { return __dsqrt_rn(a); }
     static __device__ __forceinline__ double div(double a, double b) { return __ddiv_rn(a, b); }
     static __device__ __forceinline__ double inf() { return __longlong_as_double(0x7ff0000000000000ll); }
+    static __device__ __forceinline__ double nan() { return __longlong_as_double(0x7ff8000000000000ll); }
     static __device__ __forceinline__ double sqrt_solve(double a) { return sqrt_rn64(a); }
 };
+
+// The one NaN that the sweeps work with, nan(), has a key above that of +inf, and
+// a sum with it is the same NaN.  As a value (Gamma where g is NaN) it is never
+// the smaller neighbour; as r h (nodes that keep their value: Gamma, positions
+// outside the grid) it gives a u~ that is below no value, whatever the neighbours.
+// (r h = +inf does not: with a neighbour at -inf it gives the NaN with the sign
+// set, whose key is below every value's.)
+template <class T>
+__device__ __forceinline__ T gamma_value(T g) {
+    return g == g ? g : Num<T>::nan();
+}
 
 // Wind packing: component a in {-1,0,+1} stored as (w+1) in 2 bits at 2a.
 // Sign = direction of travel: +1 when the upwind (smaller) neighbour is on the
@@ -198,8 +211,8 @@ __device__ __forceinline__ float solve2(float a, float b, float rh, bool &two) {
     return two ? u2 : u1;
 }
 // FP64: eight operations on the FP64 pipe, the comparisons, the doubling and the
-// halving on the integer pipe; in two parts like the root.  r h = +inf (fixed
-// nodes) takes the one-term branch, which gives +inf too.
+// halving on the integer pipe; in two parts like the root.  r h = +inf or NaN
+// (fixed nodes) takes the one-term branch.
 struct Solve64 {
     double ab, u1;
     Root64 root;
@@ -252,10 +265,12 @@ __device__ __forceinline__ T local_solve2(T vmx, T vpx, T vmy, T vpy, T rh, uint
     const bool lx = N::lt(vmx, vpx), ly = N::lt(vmy, vpy);
     const T a = lx ? vmx : vpx, b = ly ? vmy : vpy;
     const int sa = lx ? 1 : -1, sb = ly ? 1 : -1;
+    const bool ax = N::lt(a, b);
     bool two;
-    const T u = solve2(a, b, rh, two);
+    T u = solve2(a, b, rh, two);
+    if (!two) u = N::add(ax ? a : b, rh);  // (its own minimum differs only where a is NaN)
     wind = two ? wind_pack(sa, sb)
-               : (N::lt(u, N::inf()) ? (N::lt(a, b) ? wind_pack(sa, 0) : wind_pack(0, sb)) : WIND_ZERO);
+               : (N::lt(u, N::inf()) ? (ax ? wind_pack(sa, 0) : wind_pack(0, sb)) : WIND_ZERO);
     return u;
 }
 
@@ -328,8 +343,8 @@ __device__ __forceinline__ double div3(double x) {
 
 // Value of the 3-D local solve from the three axis minima (the same rounded
 // operations as local_solve3 on the sorted values): a sort of minima and maxima,
-// no winds.  r h = +inf (fixed nodes) gives +inf or, in FP32, NaN, and squares
-// that overflow may give NaN: neither lowers any value.
+// no winds.  r h = NaN (fixed nodes) gives NaN, and so may squares that overflow:
+// that lowers no value.
 __device__ __forceinline__ float solve3(float m0, float m1, float m2, float rh) {
     using N = Num<float>;
     const float lo = fminf(m0, m1), hi = fmaxf(m0, m1);

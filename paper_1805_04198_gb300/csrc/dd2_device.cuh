@@ -144,7 +144,7 @@ __device__ void pack_tiles_body(const DDArgs<T> &A, size_t bid, size_t nbid) {
 #pragma unroll
         for (int i = 0; i < E; ++i) {
             int xl, yl;
-            o.v[i] = Num<T>::inf();
+            o.v[i] = Num<T>::nan();
             if (skew_node<T>(e0 + i, G.tnx, G.tny, G.tnb, G.tnstepp, xl, yl)) {
                 const size_t f = (size_t)(ty * G.sy + yl) * A.sy + tx * G.sx + xl;
                 o.v[i] = FsmPolicy<T>::node(A.gamma[f] != 0, A.r[f], hs);
@@ -173,7 +173,7 @@ __device__ void pack_coarse_body(const DDArgs<T> &A, size_t bid, size_t nbid) {
         int X = d.ox + G.c * i, Y = d.oy + G.c * j;
         bool gam = A.gamma[(size_t)Y * A.sy + X] != 0;
         A.rc[a] = gam ? T(-1) : fine_at(A.r, A.sy, X, Y);
-        A.U0[a] = gam ? fine_at(A.g, A.sy, X, Y) : Num<T>::inf();
+        A.U0[a] = gam ? gamma_value(fine_at(A.g, A.sy, X, Y)) : Num<T>::inf();
         A.W[a] = WIND_ZERO;
     }
     const size_t nv = G.coarse_sk_elems / E;
@@ -190,7 +190,7 @@ __device__ void pack_coarse_body(const DDArgs<T> &A, size_t bid, size_t nbid) {
 #pragma unroll
         for (int q = 0; q < E; ++q) {
             int i, j;
-            o.v[q] = Num<T>::inf();
+            o.v[q] = Num<T>::nan();
             if (skew_node<T>(a0 - d.skoff + q, d.mx, d.my, d.nb, d.nstepp, i, j)) {
                 const size_t f = (size_t)(d.oy + G.c * j) * A.sy + d.ox + G.c * i;
                 o.v[q] = FsmPolicy<T>::node(A.gamma[f] != 0, A.r[f], Hs);
@@ -622,7 +622,7 @@ __device__ bool tile_needs_solve(const DDArgs<T> &A, int tile) {
         uint8_t wv = 0;
         size_t ca;
         if (A.gamma[(size_t)Y * A.sy + X]) {
-            v = fine_at(A.g, A.sy, X, Y);
+            v = gamma_value(fine_at(A.g, A.sy, X, Y));
         } else if (tile_inflow(A, xl, yl, X, Y, ca)) {
             v = A.U[ca];
             wv = A.W[ca];
@@ -661,13 +661,13 @@ __device__ __forceinline__ void k_fine_body(const DDArgs<T> &A, char *smem, int 
         if (xl < NX) {
             int X = tx * G.sx + xl, Y = ty * G.sy + yl;
             size_t ca;
-            if (A.gamma[(size_t)Y * A.sy + X]) v = fine_at(A.g, A.sy, X, Y);
+            if (A.gamma[(size_t)Y * A.sy + X]) v = gamma_value(fine_at(A.g, A.sy, X, Y));
             else if (tile_inflow(A, xl, yl, X, Y, ca)) v = A.U[ca];
         }
         ut[e] = v;
     }
-    // (Gamma nodes carry an infinite r h in the skewed statics, set once when
-    // the statics are packed)
+    // (the r h of Gamma nodes is NaN in the skewed statics, set once when they are
+    // packed)
     __threadfence_block();
     __syncthreads();
     // Step 3: FSM sweeps in the subdomain
@@ -744,7 +744,7 @@ __device__ __forceinline__ void k_fine_box_body(const DDArgs<T> &A, char *smem, 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const Box2<K> B(NX, NY);
     T *const su = reinterpret_cast<T *>(smem), *const sr = su + B.cells();
-    for (int i = threadIdx.x; i < 2 * B.cells(); i += blockDim.x) su[i] = INF;
+    B.clear(su, sr);
     __syncthreads();
     for (int yl = warp; yl < NY; yl += nw)
         for (int xl = lane; xl < NX; xl += 32) {
@@ -752,7 +752,7 @@ __device__ __forceinline__ void k_fine_box_body(const DDArgs<T> &A, char *smem, 
             const bool gam = A.gamma[f] != 0;
             const int q = B.at(xl, yl);
             sr[q] = FsmPolicy<T>::node(gam, A.r[f], T(G.h));
-            if (gam) su[q] = A.g[f];
+            if (gam) su[q] = gamma_value(A.g[f]);
         }
     // Step 2: boundary data.  Inflow nodes start at U, interior and outflow
     // nodes at +inf; all of them are swept (Step 3), only Gamma is fixed.

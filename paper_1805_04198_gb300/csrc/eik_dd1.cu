@@ -141,8 +141,8 @@ __device__ __forceinline__ bool group_any(bool p) {
     return ((__ballot_sync(FULL, p) >> (threadIdx.x & 31 & ~(DD1_G - 1))) & ((1u << DD1_G) - 1)) != 0;
 }
 
-// Node of a plain sweep: v = min(old, min(neighbours) + r h); r h = +inf at Gamma
-// (and where r h is no finite number), which changes nothing.  Rounding is
+// Node of a plain sweep: v = min(old, min(neighbours) + r h); r h is NaN at Gamma
+// (and where it is no finite number), which changes nothing.  Rounding is
 // monotone, so min(behind, ahead) + r h is the smaller of the two sums, and only
 // one of them is in the chain.
 template <class T>
@@ -251,7 +251,7 @@ template <class T>
 __device__ long long coarse_fsm(const DD1Args<T> &A, T *U, const T *rHc, const uint8_t *cfix, bool &conv) {
     auto load = [&](int j, FsmNode<T> &x) {
         x.old = U[j];
-        x.rh = (cfix[j] != 0) | !finite_(rHc[j]) ? Num<T>::inf() : rHc[j];
+        x.rh = (cfix[j] != 0) | !finite_(rHc[j]) ? Num<T>::nan() : rHc[j];
     };
     auto f = [](const FsmNode<T> &x, T b, T a) { return fsm_chain(fsm_rest(x.old, x.rh, a), x.rh, b); };
     auto link = [](const FsmNode<T> &x, T b) { return Num<T>::add(b, x.rh); };
@@ -332,8 +332,8 @@ __device__ int causal_rounds(int N, T *Un, const int8_t *W) {
     return rounds;
 }
 
-// A subinterval where its sweeps read and write it.  SM: u and r h (+inf where
-// fsm_chain wants it) of its M + 1 nodes and one of +inf after them in shared
+// A subinterval where its sweeps read and write it.  SM: u and r h (NaN where
+// fsm_chain wants it) of its M + 1 nodes and one that stays after them in shared
 // memory; else the interior of u, r and Gamma in global memory and the ends, which
 // two subintervals share, in `ends`.
 template <class T, bool SM>
@@ -348,7 +348,7 @@ struct Line {
     __device__ __forceinline__ T rh_at(I j) const {
         if (SM) return rh[j];
         const T v = Num<T>::mul(rh[j], h);
-        return (gm[j] != 0) | !finite_(v) ? Num<T>::inf() : v;
+        return (gm[j] != 0) | !finite_(v) ? Num<T>::nan() : v;
     }
     // position p of a sweep in direction DIR; +inf past the end
     template <int DIR>
@@ -360,7 +360,8 @@ struct Line {
             old = u[k];
             rh = this->rh[k];
         } else {
-            old = rh = Num<T>::inf();
+            old = Num<T>::inf();
+            rh = Num<T>::nan();
             if (in) {
                 old = *slot(j);
                 rh = rh_at(j);
@@ -467,8 +468,8 @@ __device__ long long solve_sub(const DD1Args<T> &A, const Line<T, SM> &L, int su
     const T *g = A.g + f0;
     const bool fix0 = gm[0] != 0, fixM = gm[M] != 0;
     const bool in0 = !fix0 && Wl > 0, inM = !fixM && Wr < 0;
-    const T s0 = fix0 ? g[0] : (in0 ? Ul : inf);
-    const T sM = fixM ? g[M] : (inM ? Ur : inf);
+    const T s0 = fix0 ? gamma_value(g[0]) : (in0 ? Ul : inf);
+    const T sM = fixM ? gamma_value(g[M]) : (inM ? Ur : inf);
     if (on) {
         for (long long j0 = 1 + lane; j0 < M; j0 += 8 * DD1_G) {
             uint8_t f[8];
@@ -476,7 +477,7 @@ __device__ long long solve_sub(const DD1Args<T> &A, const Line<T, SM> &L, int su
             for (int i = 0; i < 8; ++i) f[i] = j0 + i * DD1_G < M ? gm[j0 + i * DD1_G] : 0;
 #pragma unroll
             for (int i = 0; i < 8; ++i)
-                if (j0 + i * DD1_G < M) L.u[j0 + i * DD1_G] = f[i] ? g[j0 + i * DD1_G] : inf;
+                if (j0 + i * DD1_G < M) L.u[j0 + i * DD1_G] = f[i] ? gamma_value(g[j0 + i * DD1_G]) : inf;
         }
         if (lane == 0) {
             *L.slot(0) = s0;
@@ -550,7 +551,7 @@ __global__ void __launch_bounds__(DD1_THREADS, 1) k_dd1(DD1Args<T> A) {
         for (int i = tid; i <= N; i += nt) {
             const long long f = (long long)i * M;
             cfix[i] = A.gamma[f] ? 1 : 0;
-            U[i] = A.gamma[f] ? A.g[f] : inf;
+            U[i] = A.gamma[f] ? gamma_value(A.g[f]) : inf;
             rHc[i] = Num<T>::mul(A.r[f], A.H);
         }
         __syncthreads();
@@ -585,7 +586,7 @@ __global__ void __launch_bounds__(DD1_THREADS, 1) k_dd1(DD1Args<T> A) {
     L.gm = A.gamma + (mine ? (long long)sub * M : 0);
     if (SM) {
         const long long pitch = dd1_pitch(M);
-        // (groups past the last one only read the +inf after its nodes)
+        // (groups past the last one only read the node after its nodes)
         T *const rh = reinterpret_cast<T *>(smem + dd1_coarse_bytes<T>(N)) + (size_t)2 * min(grp, A.per - 1) * pitch;
         L.u = rh + pitch;
         L.rh = rh;
@@ -597,7 +598,10 @@ __global__ void __launch_bounds__(DD1_THREADS, 1) k_dd1(DD1Args<T> A) {
 #pragma unroll 4
             for (long long j = tid % DD1_G; j <= M; j += DD1_G) rh[j] = G.rh_at(j);
         }
-        if (grp < A.per) rh[M + 1] = L.u[M + 1] = inf;
+        if (grp < A.per) {
+            rh[M + 1] = Num<T>::nan();
+            L.u[M + 1] = inf;
+        }
         __syncthreads();
     } else {
         L.u = A.u + (mine ? (long long)sub * M : 0);
@@ -650,7 +654,7 @@ __global__ void __launch_bounds__(DD1_THREADS, 1) k_dd1(DD1Args<T> A) {
                 for (int i = tid; i <= N; i += nt) {
                     int w;
                     Cold[i] = ch1_at(U, i, N, rHc[i], w);
-                    Un[i] = cfix[i] ? A.g[(long long)i * M] : inf;
+                    Un[i] = cfix[i] ? gamma_value(A.g[(long long)i * M]) : inf;
                 }
                 __syncthreads();
                 if (tid < 32) {

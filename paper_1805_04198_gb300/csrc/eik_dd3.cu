@@ -374,12 +374,12 @@ __device__ void box3_sweeps(const Box3<T> &B, const P &pol, long long max_sweeps
     }
 }
 
-// FSM update (Sec. 1.1): u = min(u, u~), from r h (+inf at fixed nodes, whose u~
+// FSM update (Sec. 1.1): u = min(u, u~), from r h (NaN at fixed nodes, whose u~
 // is then never below their value).
 template <class T>
 struct Fsm3Update {
     using Stat = T;
-    static __device__ __forceinline__ T none() { return Num<T>::inf(); }
+    static __device__ __forceinline__ T none() { return Num<T>::nan(); }
     __device__ __forceinline__ T apply(T self, const T *vm, const T *vp, T rh, bool &changed) const {
         using N = Num<T>;
         const T ut = solve3(N::mn(vm[0], vp[0]), N::mn(vm[1], vp[1]), N::mn(vm[2], vp[2]), rh);
@@ -422,7 +422,7 @@ struct Fsm3Direct : Fsm3Update<T> {
     __device__ __forceinline__ void load_if(bool on, const Cursor &c, int ahead, T &v) const {
         if (on) {
             const long long f = c.at + ahead * c.step;
-            v = !gamma[f] && r[f] > T(0) ? Num<T>::mul(r[f], h) : Num<T>::inf();
+            v = !gamma[f] && r[f] > T(0) ? Num<T>::mul(r[f], h) : Num<T>::nan();
         }
     }
 };
@@ -443,7 +443,7 @@ struct Fsm3Grid : Fsm3Update<T> {
     __device__ __forceinline__ void load_if(bool on, const Cursor &c, int ahead, T &v) const {
         if (on) {
             const T r = rc[c.at + ahead * c.step];
-            v = r > T(0) ? Num<T>::mul(r, Hs) : Num<T>::inf();
+            v = r > T(0) ? Num<T>::mul(r, Hs) : Num<T>::nan();
         }
     }
 };
@@ -523,12 +523,12 @@ __global__ void k3_pack_coarse(DD3Args<T> A) {
         const bool gam = A.gamma[f] != 0;
         const long long a = d.off + e;
         A.rc[a] = gam ? T(-1) : A.r[f];
-        A.U0[a] = gam ? A.g[f] : Num<T>::inf();
+        A.U0[a] = gam ? gamma_value(A.g[f]) : Num<T>::inf();
         A.W[a] = WIND_ZERO;
     }
 }
 
-// r h of every subdomain in column-tile order (+inf at Gamma and outside).
+// r h of every subdomain in column-tile order (NaN at Gamma and outside).
 template <class T>
 __global__ void k3_pack_tiles(DD3Args<T> A) {
     const DD3Geom &G = A.G;
@@ -541,7 +541,7 @@ __global__ void k3_pack_tiles(DD3Args<T> A) {
     for (int e = threadIdx.x; e < n; e += blockDim.x) {
         const int lane = e & 31, row = e >> 5, ct = row / mz, z = row - ct * mz;
         const int tx = ct / nty, x = 8 * tx + (lane & 7), y = 4 * (ct - tx * nty) + (lane >> 3);
-        T v = Num<T>::inf();
+        T v = Num<T>::nan();
         if (x < mx && y < my) {
             const size_t f = fidx(A, t0 * G.S[0] + x, t1 * G.S[1] + y, t2 * G.S[2] + z);
             const T r = A.r[f];
@@ -751,7 +751,7 @@ __global__ void __launch_bounds__(BOX3_THREADS, 1) k3_fine(DD3Args<T> A) {
         T v = INF;
         uint8_t fixed = 0;
         if (A.gamma[f]) {
-            v = A.g[f];
+            v = gamma_value(A.g[f]);
             fixed = 1;
         } else if (tile3_inflow(A, l, Xg, ca)) {
             v = A.U[ca];

@@ -90,13 +90,13 @@ struct FsmArgs {
     int multi;   // multi-CTA form
 };
 
-// Skewed slowness r h (positions outside
-// the box and Gamma nodes get +inf), then the state (Sec. 1.1 initialisation:
+// Skewed slowness r h (NaN at positions
+// outside the box and Gamma nodes), then the state (Sec. 1.1 initialisation:
 // Gamma fixed at g, everything else large, padding columns included) and, for
 // the multi-CTA form, the empty hand-off columns.
 template <class T>
 __device__ void fsm_pack_body(const FsmArgs<T> &A, size_t bid, size_t nbid) {
-    skew_pack<T, 1>(A.rsk, 0, A.nx, A.ny, A.nb, A.nstepp, bid, nbid, Num<T>::inf(), [&](int, int x, int y) {
+    skew_pack<T, 1>(A.rsk, 0, A.nx, A.ny, A.nb, A.nstepp, bid, nbid, Num<T>::nan(), [&](int, int x, int y) {
         const size_t gi = (size_t)y * A.sy + x;
         return FsmPolicy<T>::node(A.gamma[gi] != 0, A.r[gi], A.h);
     });
@@ -107,7 +107,7 @@ __device__ void fsm_pack_body(const FsmArgs<T> &A, size_t bid, size_t nbid) {
         T v = Num<T>::inf();
         if (x < A.nx) {
             const size_t gi = (size_t)y * A.sy + x;
-            if (A.gamma[gi]) v = A.g[gi];
+            if (A.gamma[gi]) v = gamma_value(A.g[gi]);
         }
         A.state[t] = v;
     }
@@ -209,7 +209,7 @@ template <int K, class T>
 __device__ __forceinline__ void fsm_box_body(const FsmArgs<T> &A, char *smem, eik_fsm_stats *out) {
     const Box2<K> B(A.nx, A.ny);
     T *const su = reinterpret_cast<T *>(smem), *const sr = su + B.cells();
-    for (int i = threadIdx.x; i < 2 * B.cells(); i += blockDim.x) su[i] = Num<T>::inf();
+    B.clear(su, sr);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     for (int y = warp; y < A.ny; y += nw)
@@ -219,7 +219,7 @@ __device__ __forceinline__ void fsm_box_body(const FsmArgs<T> &A, char *smem, ei
             const T rv = A.r[gi], gv = A.g[gi];
             const int q = B.at(x, y);
             sr[q] = FsmPolicy<T>::node(gam, rv, A.h);
-            if (gam) su[q] = gv;
+            if (gam) su[q] = gamma_value(gv);
         }
     __syncthreads();
     if (warp == 0) {

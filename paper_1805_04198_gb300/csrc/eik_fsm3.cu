@@ -68,7 +68,7 @@ __global__ void k_fsm3_init(Fsm3Args<T> A) {
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
         const int x = (int)(t % A.nx), y = (int)((t / A.nx) % A.ny), z = (int)(t / ((size_t)A.nx * A.ny));
         const size_t gi = (size_t)z * A.sz + (size_t)y * A.sy + x;
-        A.w[t] = A.gamma[gi] ? A.g[gi] : Num<T>::inf();  // Sec. 1.1 initialisation
+        A.w[t] = A.gamma[gi] ? gamma_value(A.g[gi]) : Num<T>::inf();  // Sec. 1.1 initialisation
     }
     if (blockIdx.x == 0 && threadIdx.x < 4) {
         A.dev->bar[threadIdx.x] = 0;
@@ -218,18 +218,18 @@ __device__ __forceinline__ void p3_clhand(bool c, double *a, double e) {
 
 template <class T>
 __global__ void k_fsm3_pack(Fsm3Args<T> A) {
-    // state and r h, [tile][z][32]: Sec. 1.1 initialisation; +inf outside the grid
+    // state and r h, [tile][z][32]: Sec. 1.1 initialisation; +inf and NaN outside the grid
     const size_t n = (size_t)A.ntile * A.nz * 32;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
         const int p = (int)(t & 31);
         const size_t row = t >> 5;
         const int b = (int)(row / A.nz), z = (int)(row - (size_t)b * A.nz);
         const int tx = b / A.nty, x = 8 * tx + (p & 7), y = 4 * (b - tx * A.nty) + (p >> 3);
-        T v = Num<T>::inf(), rh = Num<T>::inf();
+        T v = Num<T>::inf(), rh = Num<T>::nan();
         if (x < A.nx && y < A.ny) {
             const size_t gi = (size_t)z * A.sz + (size_t)y * A.sy + x;
             const T r = A.r[gi];
-            if (A.gamma[gi]) v = A.g[gi];
+            if (A.gamma[gi]) v = gamma_value(A.g[gi]);
             else if (r > T(0)) rh = Num<T>::mul(r, A.h);
         }
         A.w[t] = v;

@@ -354,14 +354,14 @@ __device__ __forceinline__ bool wait_until(F ready, const EngineCtl &C, int swee
 }
 
 // FSM update u = min(u, u~) (Sec. 1.1, eq. FSMupdate) from the axis minima a, b.
-// Static: r h, +inf at fixed nodes (Gamma) and outside the box, whose u~ is
-// then +inf, so that they keep their value without a test.
+// Static: r h, NaN at fixed nodes (Gamma) and outside the box, whose u~ is then
+// NaN, so that they keep their value without a test.
 template <class T>
 struct FsmPolicy {
     static constexpr bool SYM = true;
     static __device__ __forceinline__ T pad() { return Num<T>::inf(); }
     static __device__ __forceinline__ T node(bool fixed, T r, T h) {
-        return !fixed && r > T(0) ? Num<T>::mul(r, h) : Num<T>::inf();
+        return !fixed && r > T(0) ? Num<T>::mul(r, h) : Num<T>::nan();
     }
     __device__ __forceinline__ T update(T self, T a, T b, T rh, bool &changed) const {
         const T ut = local_solve2_min(a, b, rh);

@@ -1,4 +1,4 @@
-"""Values at the ends of the FP64 range and signs of zero.
+"""Values at the ends of the FP64 range, signs of zero, boundary values that are no finite numbers.
 
 Against plain serial sweeps of the same closed form in numpy: where (r h)^2 overflows the discriminant of the two-term branch is +inf or, if the difference squared overflows too,
 NaN, which counts as 0; a NaN of the three-term branch leaves the node as it is."""
@@ -102,3 +102,47 @@ def test_signs_of_zero(gpu, tiles, cells, c, z, step):
         np.testing.assert_array_equal(U[on], U_ref[on])
         if step == "fine":  # the x component of its wind: from the plus side
             assert int(coarse[1][c, c]) & 3 == 0
+
+
+MINUS_NAN = np.array(0xfff8000000000000, np.uint64).view(np.float64)[()]  # what inf - inf is
+
+
+def _special(shape, v):
+    rng = np.random.default_rng(sum(shape))
+    r = rng.uniform(0.5, 2.0, shape).astype(np.float32).astype(np.float64)
+    gamma, g = np.zeros(shape, np.uint8), np.zeros(shape)
+    for k, val in enumerate((v, 0.0, 0.0625)):
+        at = tuple((s * (2 * k + 1)) // 7 for s in shape)
+        gamma[at], g[at] = 1, val
+    return r, gamma, g
+
+
+# the nodes around a NaN do as if it were not there, and it stays; -inf reaches every node
+@pytest.mark.parametrize("shape", [(11, 9), (7, 40), (4, 300), (5, 6, 11)])
+@pytest.mark.parametrize("v", [np.nan, MINUS_NAN, -np.inf, np.inf])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_special_boundary_values(gpu, shape, v, dtype):
+    r, gamma, g = _special(shape, v)
+    R, G, g_t = _dev(r, gamma, g)
+    u, st = gpu.fsm(R.to(dtype), G, g_t.to(dtype), 0.05)
+    with np.errstate(all="ignore"):
+        u_ref, n = sweeps(r, gamma, g, 0.05, 100)
+    if dtype == torch.float64:
+        np.testing.assert_array_equal(u.cpu().numpy(), u_ref)
+        assert st["sweeps"] == n
+    else:
+        np.testing.assert_allclose(u.cpu().numpy(), u_ref, rtol=1e-5, equal_nan=True)
+
+
+# subdomains of one warp and of several, 3-D boxes, the 1-D method in shared and in global memory
+@pytest.mark.parametrize("tiles,cells,c", [((2, 2), 16, 8), ((1, 2), 60, 10), ((2, 2, 2), 8, 4), ((12,), 10, 10),
+                                           ((2,), 20000, 20000)])
+@pytest.mark.parametrize("v", [np.nan, MINUS_NAN])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_special_boundary_values_dd(gpu, tiles, cells, c, v, dtype):
+    shape = tuple(t * cells + 1 for t in reversed(tiles))
+    r, gamma, g = _special(shape, v)
+    kw = dict(theta=0.2, max_iter=3, tol=0.0, max_coarse_sweeps=8)
+    R, G, g_t = _dev(r, gamma, g)
+    u, _ = gpu.dd_solve(R.to(dtype), G, g_t.to(dtype), 0.05, tiles, c, **kw)
+    np.testing.assert_array_equal(np.isnan(u.cpu().numpy()), np.isnan(g))
