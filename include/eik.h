@@ -81,7 +81,9 @@ size_t eik_fsm_workspace_size(const eik_grid *grid);
  *   gamma  [in]  Gamma mask;  g [in] boundary values, read where gamma != 0
  *   u      [out] solution (unreached nodes are +inf)
  *   ws     [in]  scratch of at least eik_fsm_workspace_size(grid) bytes,
- *                256-byte aligned; its contents need no initialisation
+ *                256-byte aligned; its contents need no initialisation (3-D
+ *                grids also run, by a slower schedule with the same result,
+ *                in one value per node and 1 kB)
  *   stats  [out] device pointer (may be NULL)
  * Returns EIK_OK, EIK_EINVAL, EIK_ENOMEM, EIK_ECUDA or EIK_EUNSUPPORTED.
  */

@@ -626,13 +626,13 @@ extern "C" int eik_profile_collect(eik_kernel_time *out, int max_entries) {
 
 namespace eik {
 // 3-D form (eik_fsm3.cu)
-size_t fsm3_workspace_size(const eik_grid *grid);
+size_t fsm3_workspace_size(const eik_grid *grid, bool least);
 int fsm3_run(const eik_grid *grid, const void *r, const uint8_t *gamma, const void *g, void *u, int64_t max_sweeps,
-             void *ws, eik_fsm_stats *stats, cudaStream_t s);
+             void *ws, size_t ws_bytes, eik_fsm_stats *stats, cudaStream_t s);
 }  // namespace eik
 
 extern "C" size_t eik_fsm_workspace_size(const eik_grid *grid) {
-    if (grid && grid->ndim == 3) return valid_grid_common(grid, 3) ? fsm3_workspace_size(grid) : 0;
+    if (grid && grid->ndim == 3) return valid_grid_common(grid, 3) ? fsm3_workspace_size(grid, false) : 0;
     FsmPlan P;
     if (!fsm_plan(grid, P)) return 0;
     return P.bytes;
@@ -654,12 +654,12 @@ extern "C" int eik_fsm(const eik_grid *grid, const void *r, const uint8_t *gamma
             set_error("workspace must be 256-byte aligned");
             return EIK_EINVAL;
         }
-        const size_t need = fsm3_workspace_size(grid);
+        const size_t need = fsm3_workspace_size(grid, true);
         if (ws_bytes < need) {
             set_error("workspace of %zu bytes is smaller than the %zu required", ws_bytes, need);
             return EIK_ENOMEM;
         }
-        return fsm3_run(grid, r, gamma, g, u, max_sweeps, ws, stats, static_cast<cudaStream_t>(stream));
+        return fsm3_run(grid, r, gamma, g, u, max_sweeps, ws, ws_bytes, stats, static_cast<cudaStream_t>(stream));
     }
     FsmPlan P;
     if (!fsm_plan(grid, P)) return EIK_EINVAL;

@@ -22,7 +22,7 @@
 //
 // k_fsm3_sweeps: hyperplanes of nodes with equal i + j + k, each updated by the
 // whole GPU, a grid barrier between them; for grids with more tiles than warps
-// fit on the GPU at once.  60 x 330 x 330 FP32: 254 ms (266 ms with the wind, which
+// fit on the GPU at once, and for workspaces without room for the tile form.  60 x 330 x 330 FP32: 254 ms (266 ms with the wind, which
 // is not needed, worked out beside the value).
 #include <algorithm>
 #include <cmath>
@@ -463,11 +463,31 @@ __global__ void k_fsm3_out(Fsm3Args<T> A, eik_fsm_stats *out) {
     }
 }
 
+// Tiles that can be co-resident on the 152 SMs (5 CTAs of k_fsm3_tiles on an SM in
+// FP32, 3 in FP64): larger grids are swept by hyperplanes, whatever the workspace.
 template <class T>
-static size_t fsm3_layout(const eik_grid *grid, Fsm3Args<T> *A, void *ws) {
+constexpr size_t T3MOST = (size_t)152 * T3WARPS * (sizeof(T) == 4 ? 5 : 3);
+
+static size_t fsm3_tile_count(const eik_grid *grid) {
+    return (size_t)((grid->n[0] + 7) / 8) * ((grid->n[1] + 3) / 4);
+}
+
+// The workspace of the tile form or of the hyperplane form, which needs the state
+// only (257^3 FP64: 136 MB; with tiles 2.5 times as much).
+template <class T>
+static size_t fsm3_layout(const eik_grid *grid, bool tiles, Fsm3Args<T> *A, void *ws) {
     const size_t ntx = (grid->n[0] + 7) / 8, nty = (grid->n[1] + 3) / 4, nt = ntx * nty;
     const size_t cells = nt * 32 * grid->n[2];
     Carver cv(ws);
+    if (!tiles) {
+        T *w = cv.take<T>((size_t)grid->n[0] * grid->n[1] * grid->n[2]);
+        Fsm3Dev *dev = cv.take<Fsm3Dev>(1);
+        if (A) {
+            A->w = w;
+            A->dev = dev;
+        }
+        return cv.used + 256;
+    }
     T *w = cv.take<T>(cells), *rp = cv.take<T>(cells);
     T *hand = cv.take<T>(nt * 12 * t3_col((int)grid->n[2]));
     int *ctl = cv.take<int>(nt + 32);
@@ -484,14 +504,19 @@ static size_t fsm3_layout(const eik_grid *grid, Fsm3Args<T> *A, void *ws) {
     return cv.used + 256;
 }
 
-size_t fsm3_workspace_size(const eik_grid *grid) {
-    return grid->dtype == EIK_F64 ? fsm3_layout<double>(grid, nullptr, nullptr)
-                                  : fsm3_layout<float>(grid, nullptr, nullptr);
+template <class T>
+static size_t fsm3_size(const eik_grid *grid, bool least) {
+    return fsm3_layout<T>(grid, !least && fsm3_tile_count(grid) <= T3MOST<T>, nullptr, nullptr);
+}
+
+// least = false: the workspace to ask for; true: what a solve can do with
+size_t fsm3_workspace_size(const eik_grid *grid, bool least) {
+    return grid->dtype == EIK_F64 ? fsm3_size<double>(grid, least) : fsm3_size<float>(grid, least);
 }
 
 template <class T>
 static int fsm3_run_t(const eik_grid *grid, const void *r, const uint8_t *gamma, const void *g, void *u,
-                      int64_t max_sweeps, void *ws, eik_fsm_stats *stats, cudaStream_t s) {
+                      int64_t max_sweeps, void *ws, size_t ws_bytes, eik_fsm_stats *stats, cudaStream_t s) {
     Fsm3Args<T> A;
     memset(&A, 0, sizeof(A));
     A.r = static_cast<const T *>(r);
@@ -505,7 +530,6 @@ static int fsm3_run_t(const eik_grid *grid, const void *r, const uint8_t *gamma,
     A.nz = (int)grid->n[2];
     A.h = (T)grid->h;
     A.max_sweeps = max_sweeps;
-    fsm3_layout<T>(grid, &A, ws);
     A.launches = 3;
     int rc, dev, nsm = 0;
     if ((rc = cuda_check(cudaGetDevice(&dev), "cudaGetDevice"))) return rc;
@@ -517,8 +541,11 @@ static int fsm3_run_t(const eik_grid *grid, const void *r, const uint8_t *gamma,
     if ((rc = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fsm3_tiles<T>, 32 * T3WARPS, 0),
                          "occupancy")))
         return rc;
-    const long long tiles = (long long)A.ntx * A.nty, ctas = (tiles + T3WARPS - 1) / T3WARPS;
-    if (ctas <= (long long)per_sm * nsm) {
+    const size_t tiles = fsm3_tile_count(grid), ctas = (tiles + T3WARPS - 1) / T3WARPS;
+    const bool tile_form = tiles <= T3MOST<T> && ctas <= (size_t)per_sm * nsm &&
+                           ws_bytes >= fsm3_layout<T>(grid, true, nullptr, nullptr);
+    fsm3_layout<T>(grid, tile_form, &A, ws);
+    if (tile_form) {
         A.ntile = (int)tiles;
         EIK_LAUNCH("fsm3_init", s, k_fsm3_pack<T><<<eb, 256, 0, s>>>(A));
         tok = prof_begin("fsm3_sweeps", s);
@@ -543,9 +570,9 @@ static int fsm3_run_t(const eik_grid *grid, const void *r, const uint8_t *gamma,
 }
 
 int fsm3_run(const eik_grid *grid, const void *r, const uint8_t *gamma, const void *g, void *u, int64_t max_sweeps,
-             void *ws, eik_fsm_stats *stats, cudaStream_t s) {
-    if (grid->dtype == EIK_F64) return fsm3_run_t<double>(grid, r, gamma, g, u, max_sweeps, ws, stats, s);
-    return fsm3_run_t<float>(grid, r, gamma, g, u, max_sweeps, ws, stats, s);
+             void *ws, size_t ws_bytes, eik_fsm_stats *stats, cudaStream_t s) {
+    if (grid->dtype == EIK_F64) return fsm3_run_t<double>(grid, r, gamma, g, u, max_sweeps, ws, ws_bytes, stats, s);
+    return fsm3_run_t<float>(grid, r, gamma, g, u, max_sweeps, ws, ws_bytes, stats, s);
 }
 
 }  // namespace eik

@@ -99,3 +99,21 @@ def test_one_dimensional_requests(lib):
     assert lib.eik_fsm_workspace_size(g) == 0
     with pytest.raises(lib.EikError, match="2-D"):
         lib.eik_dd_shard_exchange_bytes(g, lib.dd_params((10,), 100))
+
+
+@pytest.mark.parametrize("call,shape,dtype,nbytes", [
+    ("fsm", (257, 300), 0, 1978384), ("adjoint", (257, 300), 0, 10074128), ("fsm_many", (257, 300), 0, 9893632),
+    ("adjoint_many", (257, 300), 0, 50372352), ("fsm", (701, 1401), 1, 42746640), ("adjoint", (701, 1401), 1, 220442896),
+    ("fsm_many", (3, 8000), 1, 93165312), ("adjoint_many", (3, 8000), 1, 466605312), ("fsm", (60, 330, 330), 0, 52272432),
+    ("fsm", (257, 257, 257), 1, 135797296), ("fsm", (513, 513, 513), 0, 1080046128), ("fsm", (3, 430, 420), 1, 4334896)])
+def test_workspaces_do_not_grow(lib, call, shape, dtype, nbytes):
+    """A caller who keeps a workspace of the size that an earlier library asked for is not refused (five problems
+    where there are many; 3-D grids that are swept by hyperplanes)."""
+    n = list(reversed(shape)) + [1] * (3 - len(shape))
+    g = lib.Grid(len(shape), dtype, (ctypes.c_int64 * 3)(*n), (ctypes.c_int64 * 3)(1, n[0], n[0] * n[1]), 0.01)
+    so = lib.load()
+    size = {"fsm": lambda: so.eik_fsm_workspace_size(ctypes.byref(g)),
+            "fsm_many": lambda: so.eik_fsm_many_workspace_size(ctypes.byref(g), 5),
+            "adjoint": lambda: so.eik_dd_adjoint_workspace_size(ctypes.byref(g)),
+            "adjoint_many": lambda: so.eik_dd_adjoint_many_workspace_size(ctypes.byref(g), 5)}[call]()
+    assert 0 < size <= nbytes

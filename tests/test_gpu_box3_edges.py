@@ -64,3 +64,24 @@ def test_dd3_without_room_for_packed_boxes(gpu):
     got = gpu.parse_dd_stats(st)
     assert torch.equal(u, u_ref)
     assert {k: v for k, v in got.items() if k != "launches"} == {k: v for k, v in s_ref.items() if k != "launches"}
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_fsm3_in_a_workspace_without_tiles(gpu, dtype):
+    """A workspace with room for 8 bytes a node, which was once all that was asked for: the same solve."""
+    r, gamma, g = _problem((17, 21, 30), 4)
+    R, G, g_t = _dev(r, gamma, g)
+    R, g_t = R.to(dtype), g_t.to(dtype)
+    grid = gpu.make_grid(R, 0.05)
+    u_ref, s_ref = gpu.fsm(R, G, g_t, 0.05)
+    nbytes = (8 * R.numel() + 255) // 256 * 256 + 304
+    assert gpu.eik_fsm_workspace_size(grid) > nbytes
+    ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=DEV)
+    off = -ws.data_ptr() % 256
+    u = torch.empty_like(R)
+    st = torch.zeros(gpu.ctypes.sizeof(gpu.FsmStats), dtype=torch.uint8, device=DEV)
+    gpu.eik_fsm(grid, R, G, g_t, u, 1000, ws[off:off + nbytes], st)
+    torch.cuda.synchronize()
+    got = gpu.FsmStats.from_buffer_copy(bytes(st.cpu().numpy()))
+    assert torch.equal(u, u_ref)
+    assert (got.sweeps, got.converged) == (s_ref["sweeps"], 1)
