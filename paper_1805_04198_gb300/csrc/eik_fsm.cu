@@ -498,7 +498,13 @@ static int fsm_many_run(const eik_grid *grid, const FsmManyPlan &MP, int nprob, 
     cudaFuncAttributes fa;
     if ((rc = cuda_check(cudaFuncGetAttributes(&fa, k_fsmm_run<T>), "func attr"))) return rc;
     const bool single = (int)P.smem <= optin && P.nb <= 32 && regs_fit(fa, P.nb);
-    const int box_k = box2_use<T>(P.nx, P.ny);
+    // One warp a problem.  In FP64 only while the SMs have few of them: a warp that
+    // has the FP64 pipe to itself is slow, but several share it, where the engine's
+    // warps keep it full.  ms, one warp / engine: 32^2 (one column a lane) 152
+    // problems 1.23 / 1.41, 304 1.67 / 1.86, 456 2.69 / 2.39, 1200 6.04 / 4.79; 33^2
+    // (two) 152 1.88 / 1.98, 200 2.86 / 2.12, 456 5.05 / 3.02, 1200 12.2 / 6.65.
+    int box_k = box2_use<T>(P.nx, P.ny);
+    if (sizeof(T) == 8 && nprob > (box_k == 1 ? 2 : 1) * nsm) box_k = 0;
     const size_t box_smem = box2_smem_bytes<T>(P.nx, P.ny);
     const int nblk = (P.nb + P.wpc - 1) / P.wpc;
     int group = nprob;  // problems per cooperative launch

@@ -182,3 +182,16 @@ def test_dd_forward_of_many_sources(gpu):
     assert torch.isfinite(g_dd).all()
     diff = (torch.linalg.vector_norm(g_dd - g_fsm) / torch.linalg.vector_norm(g_fsm)).item()
     assert diff <= 1e-3, diff
+
+
+@pytest.mark.parametrize("shape", [(9, 30), (7, 34)])
+def test_small_fp64_grids_more_than_the_sms(gpu, shape):
+    """Small FP64 grids are swept by one warp each up to a number of problems, by the engine's warps beyond it."""
+    r = _t(np.random.default_rng(3).uniform(0.5, 2.0, shape))
+    gam, g = _sources(shape, 310, 5)
+    G, Gv = _t(gam), _t(g)
+    u, st = gpu.fsm_many(r, G, Gv, 0.05)
+    for s in range(0, 310, 31):
+        u1, s1 = gpu.fsm(r, G[s].contiguous(), Gv[s].contiguous(), 0.05)
+        assert torch.equal(u[s], u1), s
+        assert st[s]["sweeps"] == s1["sweeps"] and st[s]["converged"] == 1
