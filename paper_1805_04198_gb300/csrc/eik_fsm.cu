@@ -216,10 +216,9 @@ __device__ __forceinline__ void fsm_box_body(const FsmArgs<T> &A, char *smem, ei
         for (int x = lane; x < A.nx; x += 32) {
             const size_t gi = (size_t)y * A.sy + x;
             const bool gam = A.gamma[gi] != 0;
-            const T rv = A.r[gi], gv = A.g[gi];
             const int q = B.at(x, y);
-            sr[q] = FsmPolicy<T>::node(gam, rv, A.h);
-            if (gam) su[q] = gamma_value(gv);
+            sr[q] = FsmPolicy<T>::node(gam, A.r[gi], A.h);
+            if (gam) su[q] = gamma_value(A.g[gi]);
         }
     __syncthreads();
     if (warp == 0) {

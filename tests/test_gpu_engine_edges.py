@@ -95,3 +95,18 @@ def test_small_grids(gpu, nx, ny, dtype):
     us, sts = gpu.fsm_many(R, gs, [torch.from_numpy(g + k).to(DEV, dtype) for k in range(3)], 0.05)
     np.testing.assert_array_equal(us[0].cpu().numpy(), u)
     assert sts[0]["sweeps"] == st["sweeps"] and all(s["converged"] == 1 for s in sts)
+
+
+@pytest.mark.parametrize("shape", [(33, 30), (60, 150), (9, 8, 7)])
+def test_g_is_read_at_gamma_only(gpu, shape):
+    """The boundary values end behind the last Gamma node."""
+    r, gamma, g = _problem(shape, 5)
+    gamma[1:] = 0
+    gamma[(0,) * len(shape)] = 1
+    u_ref, _, _ = O.fsm(r, gamma, g, 0.05)
+    R, G, first = (torch.from_numpy(np.ascontiguousarray(a)).to(DEV) for a in (r, gamma, g[0]))
+    grid = gpu.make_grid(R, 0.05)
+    ws = torch.empty(gpu.eik_fsm_workspace_size(grid) + 256, dtype=torch.uint8, device=DEV)
+    u = torch.empty_like(R)
+    gpu.eik_fsm(grid, R, G, first, u, 1000, ws, None)
+    np.testing.assert_array_equal(u.cpu().numpy(), u_ref)
