@@ -504,6 +504,16 @@ static int fsm_many_run(const eik_grid *grid, const FsmManyPlan &MP, int nprob, 
     // (two) 152 1.88 / 1.98, 200 2.86 / 2.12, 456 5.05 / 3.02, 1200 12.2 / 6.65.
     int box_k = box2_use<T>(P.nx, P.ny);
     if (sizeof(T) == 8 && nprob > (box_k == 1 ? 2 : 1) * nsm) box_k = 0;
+    // (a problem reads all of its own before it writes u, but others read then too)
+    if (box_k && nprob > 1) {
+        std::vector<Span> spans = {grid_span(r, grid, sizeof(T), nprob, false)};
+        for (int p = 0; p < nprob; ++p) {
+            spans.push_back(grid_span(gamma[p], grid, 1, p, false));
+            spans.push_back(grid_span(g[p], grid, sizeof(T), p, false));
+            spans.push_back(grid_span(u[p], grid, sizeof(T), p, true));
+        }
+        if (outputs_meet_inputs(spans)) box_k = 0;
+    }
     const size_t box_smem = box2_smem_bytes<T>(P.nx, P.ny);
     const int nblk = (P.nb + P.wpc - 1) / P.wpc;
     int group = nprob;  // problems per cooperative launch

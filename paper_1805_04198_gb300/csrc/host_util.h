@@ -2,10 +2,12 @@
 // carving, launch checks).
 #pragma once
 
+#include <algorithm>
 #include <cstdarg>
 #include <cstddef>
 #include <cstdint>
 #include <cstdio>
+#include <vector>
 
 #include <cuda_runtime.h>
 
@@ -39,6 +41,42 @@ inline cudaError_t set_dyn_smem(F *func, int bytes) {
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute((const void *)func, cudaFuncAttributePreferredSharedMemoryCarveout,
                                 (int)cudaSharedmemCarveoutMaxShared);
+}
+
+// The bytes of an array laid out as a grid, and the problem that it belongs to.
+struct Span {
+    uintptr_t begin, end;
+    int owner;
+    bool out;
+};
+inline Span grid_span(const void *p, const eik_grid *g, size_t elem, int owner, bool out) {
+    size_t n = (size_t)g->n[0];
+    for (int a = 1; a < g->ndim; ++a) n += (size_t)(g->n[a] - 1) * (size_t)g->stride[a];
+    const uintptr_t b = reinterpret_cast<uintptr_t>(p);
+    return Span{b, b + n * elem, owner, out};
+}
+
+// Whether an output shares memory with an input of another owner: asked where some
+// blocks read the caller's arrays while others already write outputs.
+inline bool outputs_meet_inputs(std::vector<Span> &v) {
+    std::sort(v.begin(), v.end(), [](const Span &a, const Span &b) { return a.begin < b.begin; });
+    // of the spans before: the furthest end of an output and of an input, and the
+    // furthest of another owner than that one's
+    Span far[2][2] = {};
+    for (Span &f : far[0]) f.owner = -1;
+    for (Span &f : far[1]) f.owner = -1;
+    for (const Span &s : v) {
+        for (const Span &f : far[s.out ? 0 : 1])
+            if (f.owner >= 0 && f.owner != s.owner && f.end > s.begin) return true;
+        Span *f = far[s.out ? 1 : 0];
+        if (f[0].owner == s.owner || s.end > f[0].end) {
+            if (f[0].owner != s.owner) f[1] = f[0];
+            if (f[0].owner != s.owner || s.end > f[0].end) f[0] = s;
+        } else if (f[1].owner < 0 || s.end > f[1].end) {
+            f[1] = s;
+        }
+    }
+    return false;
 }
 
 inline int cuda_check(cudaError_t e, const char *what) {
