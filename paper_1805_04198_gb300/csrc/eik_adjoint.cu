@@ -214,10 +214,6 @@ __device__ void adj_run_global_body(const AdjArgs<T> &A, char *smem, int cta) {
     long long sweeps;
     bool conv;
     engine_run<T, 5, false, true>(bx, pol, A.max_sweeps, smem, sweeps, conv, &A.dev->err, A.ghands, A.gctl, cta);
-    if (cta == 0 && threadIdx.x == 0) {
-        A.dev->sweeps = (unsigned long long)sweeps;
-        A.dev->converged = conv ? 1 : 0;
-    }
 }
 
 template <class T>
@@ -236,8 +232,11 @@ __device__ void adj_grad_body(const AdjArgs<T> &A, eik_adjoint_stats *out, size_
         }
     }
     if (out && bid == 0 && threadIdx.x == 0) {
-        out->sweeps = (int64_t)A.dev->sweeps;
-        out->converged = A.dev->converged;
+        long long sweeps = (long long)A.dev->sweeps;
+        bool conv = A.dev->converged != 0;
+        if (A.multi) engine_result(A.gctl, A.max_sweeps, sweeps, conv);
+        out->sweeps = sweeps;
+        out->converged = conv ? 1 : 0;
         out->error = A.dev->err;
         out->launches = A.launches;
     }

@@ -169,10 +169,6 @@ __device__ void fsm_run_global_body(const FsmArgs<T> &A, char *smem, int cta) {
     long long sweeps;
     bool conv;
     engine_run<T, 1, false, true>(bx, pol, A.max_sweeps, smem, sweeps, conv, &A.dev->err, A.ghands, A.gctl, cta);
-    if (cta == 0 && threadIdx.x == 0) {
-        A.dev->sweeps = (unsigned long long)sweeps;
-        A.dev->converged = conv ? 1 : 0;
-    }
 }
 
 template <class T>
@@ -189,10 +185,13 @@ __device__ void fsm_unpack_body(const FsmArgs<T> &A, eik_fsm_stats *out, size_t 
         A.u[(size_t)y * A.sy + x] = A.state[box_index(x, y, A.ny)];
     }
     if (out && bid == 0 && threadIdx.x == 0) {
-        out->sweeps = (int64_t)A.dev->sweeps;
-        out->converged = A.dev->converged;
+        long long sweeps = (long long)A.dev->sweeps;
+        bool conv = A.dev->converged != 0;
+        if (A.multi) engine_result(A.gctl, A.max_sweeps, sweeps, conv);
+        out->sweeps = sweeps;
+        out->converged = conv ? 1 : 0;
         out->error = A.dev->err;
-        out->updates = (int64_t)A.dev->sweeps * A.nx * A.ny;
+        out->updates = sweeps * A.nx * A.ny;
         out->launches = A.launches;
     }
 }

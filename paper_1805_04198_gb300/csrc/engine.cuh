@@ -713,6 +713,17 @@ __device__ int run_block(const Box<T, NST> &bx, const P &pol, int k, int b, cons
     return __any_sync(FULL, changed) ? 1 : 0;
 }
 
+// What a run ended with, from its control words.  Final in the kernel itself only
+// with one CTA: of several, the last to finish a sweep that was the last allowed may
+// find that it changed nothing when the others have left already, so their result is
+// read in a later kernel.
+__device__ __forceinline__ void engine_result(const int *ctl, long long max_sweeps, long long &sweeps,
+                                              bool &converged) {
+    const int st = vload(ctl + 1);
+    converged = st != 0x7fffffff && !vload(ctl);
+    sweeps = st != 0x7fffffff ? (long long)st + 1 : max_sweeps;
+}
+
 // Runs sweeps on one box until a sweep changes nothing or max_sweeps ran.
 // Single-CTA form (GLOBAL = false): the CTA holds every block of the box,
 // blockDim.x >= 32 * bx.nb, engine_smem_bytes<T, NST, HASB>(nb, ny) bytes of
@@ -797,9 +808,7 @@ __device__ void engine_run(const Box<T, NST> &bx, const P &pol, long long max_sw
         }
     }
     __syncthreads();
-    const int st = vload(C.stop_at);
-    converged = st != 0x7fffffff && !vload(C.abort_flag);
-    sweeps = st != 0x7fffffff ? (long long)st + 1 : max_sweeps;
+    engine_result(ints, max_sweeps, sweeps, converged);
     __syncthreads();
 }
 

@@ -110,3 +110,23 @@ def test_g_is_read_at_gamma_only(gpu, shape):
     u = torch.empty_like(R)
     gpu.eik_fsm(grid, R, G, first, u, 1000, ws, None)
     np.testing.assert_array_equal(u.cpu().numpy(), u_ref)
+
+
+@pytest.mark.parametrize("shape", [(40, 300), (24, 1100)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_converged_in_the_last_sweep_allowed(gpu, shape, dtype):
+    """Grids swept by several thread blocks, with exactly the sweeps that they need and with one less."""
+    r, gamma, g = _problem(shape, 8)
+    R, G, g_t = torch.from_numpy(r).to(DEV, dtype), torch.from_numpy(gamma).to(DEV), torch.from_numpy(g).to(DEV, dtype)
+    u, st = gpu.fsm(R, G, g_t, 0.05)
+    d = torch.ones_like(R)
+    grad, ast = gpu.adjoint(R, G, u, d, 0.05)
+    n, m = st["sweeps"], ast["sweeps"]
+    many = [gpu.fsm_many(R, [G] * 3, [g_t] * 3, 0.05, max_sweeps=n + k)[1] for k in (-1, 0)]
+    assert [[s["converged"] for s in q] for q in many] == [[0] * 3, [1] * 3]
+    for _ in range(25):
+        for k, conv in ((-1, 0), (0, 1)):
+            s = gpu.fsm(R, G, g_t, 0.05, max_sweeps=n + k)[1]
+            assert (s["sweeps"], s["converged"]) == (n + k, conv)
+            s = gpu.adjoint(R, G, u, d, 0.05, max_sweeps=m + k)[1]
+            assert (s["sweeps"], s["converged"]) == (m + k, conv)
