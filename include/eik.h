@@ -413,8 +413,9 @@ int eik_profile_collect(eik_kernel_time *out, int max_entries);
  * cooperative kernels; an expired wait records EIK_EDEVICE_TIMEOUT in the
  * call's device statistics (eik_dd_stats.error, eik_fsm_stats.error, ...),
  * makes the rest of that call return early, and never traps, so the context
- * stays usable.  Each poll sleeps 32 ns to 1 us.  0 restores the default of
- * 2^22 polls (seconds).  A small limit makes ordinary waits expire: it exists
+ * stays usable.  Each poll sleeps 32 ns to 1 us; the waits of a 2-D sweep, which
+ * sleep 256 ns at most, make four polls for one of the limit.  0 restores the
+ * default of 2^22 polls (seconds).  A small limit makes ordinary waits expire: it exists
  * to test the timeout path.  It applies to work enqueued after it returns
  * (it is a cudaMemcpyToSymbol, ordered against the legacy default stream);
  * do not change it while a call is running.  No counterpart in the paper.

@@ -760,7 +760,9 @@ __device__ void engine_run(const Box<T, NST> &bx, const P &pol, long long max_sw
     M.sbring = (unsigned)__cvta_generic_to_shared(p_sb + (size_t)warp * sb_b);
     M.halo = (unsigned)__cvta_generic_to_shared(p_small + (size_t)warp * small_b);
     EngineCtl C;
-    C.lim = spin_limit();
+    // polls here sleep 256 ns at most, a quarter of what the limit counts with
+    const long long lim = spin_limit();
+    C.lim = lim < (1ll << 60) ? 4 * lim : lim;
     C.abort_flag = ints;
     C.stop_at = ints + 1;
     C.fin = ints + 8;

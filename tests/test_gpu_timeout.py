@@ -72,3 +72,17 @@ def test_fsm_multi_cta_expired_wait_reports_timeout_then_solves_exactly():
     u_ref, sweeps, conv = oracle.fsm(r, gamma, g, h)
     assert np.array_equal(u2.cpu().numpy(), u_ref)
     assert st2["sweeps"] == sweeps
+
+
+@pytest.mark.parametrize("dtype,limit", [(torch.float64, 600), (torch.float32, 100)])
+def test_limits_that_ordinary_waits_keep(dtype, limit):
+    """The longest wait of a 257 x 257 grid in one thread block (the last warp's for the first row of a sweep) has
+    always been within these limits: a shorter sleep between polls must not make it expire."""
+    r, gamma, g, h = _case()
+    rd, gd, vd = _dev(r, gamma, g)
+    eik.eik_set_wait_limit(limit)
+    try:
+        _, st = eik.fsm(rd.to(dtype), gd, vd.to(dtype), h)
+    finally:
+        eik.eik_set_wait_limit(0)
+    assert st["error"] == 0 and st["converged"] == 1
