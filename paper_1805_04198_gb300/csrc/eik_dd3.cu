@@ -292,7 +292,9 @@ __device__ void box3_sweeps(const Box3<T> &B, const P &pol, long long max_sweeps
 #pragma unroll
             for (int i = 0; i < 4; ++i) nb[t][i] = INF;
             sa[t] = sb[t] = P::none();
-            pc[t] = pol.cursor(cv[t] ? cx[t] : 0, cv[t] ? cy[t] : 0, warp * BOX3_SLOTS + t, lane, z0, sz, -base);
+            // (a lane without a column has no place to count from)
+            pc[t] = pol.cursor(cv[t] ? cx[t] : 0, cv[t] ? cy[t] : 0, warp * BOX3_SLOTS + t, lane, z0, sz,
+                               cv[t] ? -base : 0);
             pol.load_if((unsigned)kp[t] < (unsigned)mz, pc[t], 0, sa[t]);
             pol.load_if((unsigned)(kp[t] + 1) < (unsigned)mz, pc[t], 1, sb[t]);
             if (base == 0) cur[t] = su[B.at(cx[t], cy[t], z0)];  // a lane on its first node at hyperplane 0
