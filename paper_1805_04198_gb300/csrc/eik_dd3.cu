@@ -132,8 +132,9 @@ __device__ __forceinline__ int coarse_axes3(int X, int Y, int Z, int c) {
 constexpr int BOX3_SLOTS = 2;      // tiles per warp with prefetched data
 constexpr int BOX3_THREADS = 768;  // threads of a box-sweep CTA
 
-// The box (mx x my x mz) that decides whether a size is supported: an upper
-// bound of the shared memory taken.
+// The shared memory by which a box (mx x my x mz) is accepted or refused: the
+// documented size limit.  The bordered layout may take more, up to what
+// box3_pitch is given, the layout without border takes less.
 __host__ inline size_t box3_limit(int mx, int my, int mz, size_t tsz) {
     return (size_t)mz * (mx * my + ((mx * my) & 1)) * (tsz + 1) + 16;
 }
@@ -1331,9 +1332,10 @@ static int dd3_run_t(const eik_grid *grid, const void *r, const uint8_t *gamma, 
     if ((rc = cuda_check(cudaGetDevice(&dev), "cudaGetDevice"))) return rc;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if ((int)P.fine_limit > optin || (int)P.grid_limit > optin) {
-        set_error("3-D subdomain or coarse grid box needs %zu / %zu bytes of shared memory (limit %d)", P.fine_limit,
-                  P.grid_limit, optin);
+    if ((int)P.fine_limit > optin || (int)P.grid_limit > optin || (int)P.fine_smem > optin ||
+        (int)P.grid_smem > optin) {
+        set_error("3-D subdomain or coarse grid box needs %zu / %zu bytes of shared memory (limit %d)",
+                  std::max(P.fine_limit, P.fine_smem), std::max(P.grid_limit, P.grid_smem), optin);
         return EIK_EUNSUPPORTED;
     }
     void (*const fine)(DD3Args<T>) = lean ? k3_fine<T, false> : k3_fine<T, true>;
