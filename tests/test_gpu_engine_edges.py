@@ -77,6 +77,21 @@ def test_small_boxes_f32(gpu, nx, ny, c):
     assert st["fsm_sweeps_max"] == st_ref["sweeps"]
 
 
+# ... and the same against the engine: the plain solve is made too wide for the one-warp form by a strip of Gamma nodes
+# at +inf, which changes nothing
+@pytest.mark.parametrize("nx,ny,c", [(3, 3, 2), (17, 9, 8), (32, 32, 31), (33, 5, 2), (64, 22, 21), (96, 20, 19), (97, 33, 32),
+                                     (127, 97, 6)])
+def test_small_boxes_f32_against_the_engine(gpu, nx, ny, c):
+    r, gamma, g = _problem((ny, nx), nx + 3 * ny)
+    wide = [np.concatenate([a, np.full((ny, 140), v, a.dtype)], 1) for a, v in ((r, 1.0), (gamma, 1), (g, np.inf))]
+    u_ref, st_ref = _fsm(gpu, *wide, 0.05, torch.float32)
+    u, st = gpu.dd_solve(torch.from_numpy(r).to(DEV, torch.float32), torch.from_numpy(gamma).to(DEV),
+                         torch.from_numpy(g).to(DEV, torch.float32), 0.05, (1, 1), c, max_iter=2)
+    off = (np.arange(ny)[:, None] % c != 0) & (np.arange(nx)[None, :] % c != 0)
+    np.testing.assert_array_equal(u.cpu().numpy()[off], u_ref[:, :nx][off])
+    assert st["fsm_sweeps_max"] == st_ref["sweeps"]
+
+
 # plain sweeping of a small grid takes the one-warp form up to 128 (FP64: 36) columns while the box fits an SM; one by
 # itself and several in a call, against the same nodes inside a grid too wide for it: a strip of Gamma nodes at +inf
 # beside them changes nothing
