@@ -77,7 +77,8 @@ size_t eik_fsm_workspace_size(const eik_grid *grid);
  * -1 first), with the update u = min(u, u~).  Gamma nodes are fixed at g; all
  * other nodes start at +inf.  Stops after the first sweep that changes no value
  * (the discrete solution) or after max_sweeps sweeps.
- *   r      [in]  slowness, > 0 and finite at every non-Gamma node
+ *   r      [in]  slowness, > 0 and finite at every non-Gamma node (in FP32 with
+ *                r h between 1e-19 and 1e19, whose squares FP32 holds)
  *   gamma  [in]  Gamma mask;  g [in] boundary values, read where gamma != 0
  *   u      [out] solution (unreached nodes are +inf)
  *   ws     [in]  scratch of at least eik_fsm_workspace_size(grid) bytes,

@@ -2,9 +2,10 @@
 // baseline the domain decomposition is compared against, plus the shared host
 // helpers of the C ABI (error text, version).
 //
-// The grid is one box for the warp-systolic engine: one warp per 32-column
-// block, all blocks of the grid in one CTA, sweeps cycling through the four
-// orderings until a sweep changes nothing.
+// Sweeps cycle through the four orderings until one changes nothing.  Small grids
+// are swept by one warp in shared memory, in one launch (box2.cuh).  Larger ones
+// are one box for the warp-systolic engine, one warp per 32-column block: all
+// blocks in one CTA up to MAX_SINGLE_NB, else spread over co-resident CTAs.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -254,8 +255,10 @@ constexpr void (*fsm_box_kernel(int k))(FsmArgs<T>, eik_fsm_stats *) {
 
 // Widest grid (32-column blocks) swept by one CTA.  Above it the blocks' warps
 // share too few schedulers and spreading them over CTAs wins in spite of the
-// slower hand-off (FP32 us a sweep, one CTA / several: 257^2 50.6 / 51.2,
-// 513^2 114 / 97; FP64 129^2 171 / 179, 257^2 335 / 324).
+// slower hand-off, which counts most where a grid has few rows.  ms a solve, one
+// CTA / several: FP32 257^2 3.55 / 3.36 and 20 x 257 1.74 / 1.92, 289^2 4.27 / 4.10
+// and 20 x 289 2.07 / 2.24, 353^2 6.15 / 5.48 and 20 x 353 2.99 / 2.82; FP64 161^2
+// 8.72 / 8.99, 257^2 21.5 / 20.1 and 20 x 280 9.88 / 10.3.
 constexpr int MAX_SINGLE_NB = 9;
 
 struct FsmPlan {
