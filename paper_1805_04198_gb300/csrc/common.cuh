@@ -223,12 +223,11 @@ __device__ __forceinline__ Solve64 solve2_start(double a, double b, double rh) {
     Solve64 S;
     const double d = N::sub(a, b);
     S.two = N::within(d, rh) && __double2hiint(rh) < 0x7ff00000;
-    // 2 r h by its exponent (exact, +inf above the range; where r h is subnormal
-    // its square is 0 in any case).  Not 2 (r h)^2: that loses the bits of a square
-    // just below the normal range.
-    const int rhi = __double2hiint(rh);
-    const bool top = rhi >= 0x7fe00000;
-    const double rh2 = __hiloint2double(top ? 0x7ff00000 : rhi + (1 << 20), top ? 0 : __double2loint(rh));
+    // 2 r h by its exponent (exact; where r h is subnormal its square is 0 in any
+    // case; above the range another number whose product with r h is +inf too).
+    // Not 2 (r h)^2: that loses the bits of a square just below the normal range.
+    const unsigned rhi = (unsigned)__double2hiint(rh) + (1u << 20);
+    const double rh2 = __hiloint2double((int)min(rhi, 0x7fefffffu), __double2loint(rh));
     const double disc = N::sub(N::mul(rh2, rh), N::mul(d, d));
     S.root = root_start(S.two ? disc : 1.0);
     S.ab = N::add(a, b);
