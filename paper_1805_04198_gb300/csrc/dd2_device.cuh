@@ -752,7 +752,7 @@ __device__ __forceinline__ void k_fine_box_body(const DDArgs<T> &A, char *smem, 
             const bool gam = A.gamma[f] != 0;
             const int q = B.at(xl, yl);
             sr[q] = FsmPolicy<T>::node(gam, A.r[f], T(G.h));
-            if (gam) su[q] = gamma_value(A.g[f]);
+            if (gam) su[q] = box2_gamma(A.g[f]);
         }
     // Step 2: boundary data.  Inflow nodes start at U, interior and outflow
     // nodes at +inf; all of them are swept (Step 3), only Gamma is fixed.

@@ -218,7 +218,7 @@ __device__ __forceinline__ void fsm_box_body(const FsmArgs<T> &A, char *smem, ei
             const bool gam = A.gamma[gi] != 0;
             const int q = B.at(x, y);
             sr[q] = FsmPolicy<T>::node(gam, A.r[gi], A.h);
-            if (gam) su[q] = gamma_value(A.g[gi]);
+            if (gam) su[q] = box2_gamma(A.g[gi]);
         }
     __syncthreads();
     if (warp == 0) {
