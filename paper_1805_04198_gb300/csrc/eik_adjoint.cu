@@ -284,7 +284,7 @@ static bool adj_plan(const eik_grid *grid, AdjPlan &P) {
     P.nx = (int)grid->n[0];
     P.ny = (int)grid->n[1];
     P.nb = ceil32(P.nx);
-    P.nstepp = nstep_padded(P.ny);
+    P.nstepp = nstep_whole_grid(P.ny);
     P.wpc = 2;
     const bool f64 = grid->dtype == EIK_F64;
     P.smem = f64 ? engine_smem_bytes<double, 5, false>(P.nb, P.ny) : engine_smem_bytes<float, 5, false>(P.nb, P.ny);

@@ -291,7 +291,7 @@ static bool fsm_plan(const eik_grid *grid, FsmPlan &P) {
     P.nx = (int)grid->n[0];
     P.ny = (int)grid->n[1];
     P.nb = ceil32(P.nx);
-    P.nstepp = nstep_padded(P.ny);
+    P.nstepp = nstep_whole_grid(P.ny);
     P.smem = grid->dtype == EIK_F64 ? engine_smem_bytes<double, 1, false>(P.nb, P.ny)
                                      : engine_smem_bytes<float, 1, false>(P.nb, P.ny);
     // FP64: one warp per CTA, each with an SM's FP64 pipe of its own (two warps

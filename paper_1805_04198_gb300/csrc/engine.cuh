@@ -72,9 +72,12 @@ __host__ __device__ inline size_t box_index(int i, int j, int my) {
     return ((size_t)(i >> 5) * my + j) * 32 + (i & 31);
 }
 
-// Steps of one statics stream, padded to whole chunks plus the lead (two chunks
-// ahead of the last).
-__host__ __device__ inline int nstep_padded(int ny) { return ((ny + 31 + CH - 1) / CH) * CH + 3 * CH; }
+// Steps of one statics stream, padded to whole chunks plus at least the lead (two
+// chunks ahead of the last).  Plain sweeping and the adjoint take a chunk less than
+// the decomposition: that makes room for their hand-off columns in the workspace
+// sizes that callers know.
+__host__ __device__ inline int nstep_padded(int ny) { return ((ny + 31 + CH - 1) / CH) * CH + 4 * CH; }
+__host__ __device__ inline int nstep_whole_grid(int ny) { return nstep_padded(ny) - CH; }
 
 // Sweep direction d in [0, 4): bit 1 = sign of x, bit 0 = sign of y (set =
 // +1).  The paper's loop nest (x sign outermost, -1 first) visits d = 0..3 in
